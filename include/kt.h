@@ -125,8 +125,10 @@ typedef struct {
     int block_warps;         /* warps per block, 0 = automatic                   (0) */
     int blocks_per_sm;       /* persistent grid = blocks_per_sm x SMs, 0 = automatic (0) */
     int use_graph;           /* 1: kt_integrate replays a captured CUDA graph    (0) */
-    int cells_per_warp;      /* 32: one cell per lane (networks with <= 16 unknowns);
-                                1: one cell per warp (<= 96 unknowns); 0: automatic (0) */
+    int cells_per_warp;      /* 32: the small-network kernels (<= 16 unknowns), one cell
+                                per lane or, where that is faster, per group of lanes
+                                (the same results bit for bit); 1: the large-network
+                                kernels, a cell per warp (<= 96 unknowns); 0: automatic (0) */
     int schedule;            /* kt_integrate on a state with persistent = 1: 1 hands
                                 out the cells with the most Newton iterations in the
                                 previous call first (the state's n_newton counters;

@@ -71,6 +71,10 @@ struct kt_network {
     std::vector<double> tab;                      // [ntab][nR][nT] ln k
     std::vector<unsigned char> blob;
     NetView view{};
+    // programs of the kernels with 4, 8, 16 or 32 lanes per cell (FP64 form, then FP32-LU):
+    // they follow the tables (view.bytes_total) in the blob; -1 where the network has none
+    std::array<int, 8> coop_off{{-1, -1, -1, -1, -1, -1, -1, -1}};
+    std::array<kt::CoopTab, 8> coop_tab{};
     const kt_mlp *mlp = nullptr;                  // attached learned-guess MLP (not owned)
     std::mutex mu;
     std::map<int, unsigned char *> dev_blob;      // device ordinal -> device copy
@@ -417,6 +421,24 @@ void build_blob(kt_network *n)
     }
 }
 
+// Appends the per-lane programs of every group size to the blob.
+void build_coop(kt_network *n)
+{
+    if (n->ns + n->energy > kt::kLaneMaxN || n->view.special) return;
+    std::vector<unsigned char> prog;
+    std::vector<double> dH(n->nr);
+    std::memcpy(dH.data(), n->blob.data() + n->view.off_dH, 8 * dH.size());
+    for (int i = 0; i < 8; ++i) {
+        if (!kt::coop_tables(n->view.N, n->ns, n->nr, n->energy, n->nin.data(), n->nout.data(),
+                             reinterpret_cast<const int(*)[kt::kMaxSide]>(n->in.data()),
+                             reinterpret_cast<const int(*)[kt::kMaxSide]>(n->out.data()), dH.data(), i >= 4,
+                             4 << (i & 3), &n->coop_tab[i], &prog))
+            return;
+        n->coop_off[i] = static_cast<int>(n->blob.size());
+        n->blob.insert(n->blob.end(), prog.begin(), prog.end());
+    }
+}
+
 int check_opts(const kt_options *o)
 {
     if (!o) return fail(KT_EINVAL, "options: NULL");
@@ -498,6 +520,7 @@ int kt_network_load(const char *path, kt_network **out)
         return rc;
     }
     build_blob(n);
+    build_coop(n);
     *out = n;
     return KT_OK;
 }
@@ -614,7 +637,17 @@ int integrate_impl(const kt_network *net, int64_t ncells, const double *y_in, co
     a.scratch = static_cast<kt::Scratch *>(scratch);
     a.order = opts->persistent ? order : nullptr;
     kt::LaunchCfg c{opts->form, opts->persistent, opts->block_warps, opts->blocks_per_sm, cpw, opts->lane_variant};
-    int ce = cpw == 32 ? kt::launch_lane(a, c, cuda_stream) : kt::launch_warp(a, c, cuda_stream);
+    a.persistent = opts->persistent != 0;
+    const int grp = cpw == 32 ? kt::coop_group(a, c) : 0;
+    const int gi = (grp == 4 ? 0 : (grp == 8 ? 1 : (grp == 16 ? 2 : 3))) + (opts->form == KT_FORM_FP32LU ? 4 : 0);
+    if (grp && net->coop_off[gi] >= 0) {
+        a.coop = blob + net->coop_off[gi];
+        a.coop_tab = net->coop_tab[gi];
+        a.coop_g = grp;
+        if (!kt::coop_fits(a, c)) a.coop = nullptr;
+    }
+    int ce = a.coop ? kt::launch_coop(a, c, cuda_stream)
+                    : cpw == 32 ? kt::launch_lane(a, c, cuda_stream) : kt::launch_warp(a, c, cuda_stream);
     if (ce != 0) return cuda_fail(static_cast<cudaError_t>(ce), "integrate kernel launch");
     return KT_OK;
 }

@@ -3,6 +3,7 @@
 
 #include <cstdint>
 #include <cstddef>
+#include <vector>
 
 #include "../../include/kt.h"
 
@@ -74,9 +75,42 @@ struct Scratch {
 
 enum DevError : int { kDevErrNone = 0, kDevErrTma = 1 };
 
+// Per-lane programs of the kernels that give a cell G lanes (kt_coop.cuh), laid out by
+// kt_coop_tables.cu for one network and group size: which components a lane owns, the
+// terms of the f rows it sums and of the matrix entries it assembles, in the order in
+// which the lane-per-cell kernels add them.
+// A row term holds the byte offsets of its rate (bits 0..13) and of its coefficient (16..31:
+// +1, -1 or minus the reaction's heat); a matrix term those of its partial derivative (0..13)
+// and of its coefficient (16..29: +1, -1 or the heat over C_V) in the cell's partials.
+constexpr unsigned kCoopOffset = 0x3fffu;
+constexpr unsigned kCoopEnd = 1u << 15;     // last term of a row or entry
+constexpr unsigned kCoopDiag = 1u << 14;    // ... whose entry is on the diagonal
+constexpr int kCoopConst = 4;               // 0, 1, -1 before the partials
+constexpr int kCoopMaxReactions = 400;    // offsets stay within 14 bits (5 kinds x 8 bytes)
+constexpr int kCoopPad = 2;                 // padding steps after each program (prefetch)
+// Compile-time size classes (3, 11, any) and row stride of the cell's matrix: rows start on
+// 16 bytes so the solve reads four FP32 factors at a time.
+constexpr int coop_nm(int N) { return N == 3 ? 3 : (N == 11 ? 11 : kLaneMaxN); }
+constexpr int coop_ld(int NM) { return (NM + 3) & ~3; }
+constexpr int kCoopMaxWarps = 4;
+
+struct CoopTab {
+    int n_row, n_jac;      // steps of the row and matrix programs
+    int off_row, off_jac;  // byte offsets of the uint32 [step][G] programs (the owned
+                           // components, int8 [G][NC], come first)
+    int off_to, off_coef;  // matrix places uint8 [k][G] of each lane's k-th entry; row
+                           // coefficients, double: 0, 1, -1, -dH_r
+    int nin_max;           // largest number of reactants
+    int bytes;             // multiple of 16
+};
+
 struct LaunchArgs {
     NetView nv;
     const unsigned char *blob;   // device network blob
+    const unsigned char *coop;   // device programs of the chosen group size (null: one cell per lane)
+    CoopTab coop_tab;
+    int coop_g;                  // lanes per cell of those programs
+    int persistent;
     DevOpts o;
     double dt;
     const double *dt_cell;       // per-cell dt (device, may be null: dt for every cell)
@@ -184,6 +218,39 @@ inline LaneLayout lane_layout_lean(int N, int nr, int energy, int blob_bytes, in
     return L;
 }
 
+// Shared memory of the kernels with G lanes per cell: the staged network, the programs,
+// two barriers, then one region per cell.  The cell stride is an odd multiple of 16 bytes,
+// so the cells of a warp start 4 banks apart and the broadcasts of 8 cells do not collide.
+struct CoopLayout {
+    CoopTab tab;
+    int off_tab, off_bar, base, cell_bytes, groups;
+    int off_F, off_YF, off_W, off_K, off_CV, off_P, off_M, off_V, off_X;
+};
+
+inline CoopLayout coop_layout(int N, int nr, int energy, int fp32, int blob_bytes, int cvpoly, const CoopTab &tab)
+{
+    CoopLayout L{};
+    L.tab = tab;
+    L.off_tab = (blob_bytes + 15) & ~15;
+    L.off_bar = L.off_tab + tab.bytes;
+    L.base = (L.off_bar + 16 + 127) & ~127;
+    const int r = fp32 ? 4 : 8;
+    int o = 0;
+    auto take = [&](int bytes) { const int at = o; o = (o + bytes + 15) & ~15; return at; };
+    take(N * 8);                                  // iterate
+    L.off_F = take(N * 8);
+    L.off_YF = fp32 ? take(N * 4) : 0;
+    L.off_W = take((nr + 1) * 8);
+    L.off_K = energy ? 0 : take(nr * 8);
+    L.off_CV = cvpoly ? take(10 * 8) : 0;
+    L.off_P = take((kCoopConst + nr * (tab.nin_max + (energy ? 2 : 0))) * r);
+    L.off_M = take(N * coop_ld(coop_nm(N)) * r);
+    L.off_V = take(N * r);
+    L.off_X = take(coop_ld(coop_nm(N)) * r);
+    L.cell_bytes = ((o / 16) | 1) * 16;
+    return L;
+}
+
 // Shared-memory layout of one warp of the warp-per-cell kernels (one cell per warp).
 // Matrices are row-major with an odd row stride NP (conflict-free column reads).
 struct WarpLayout {
@@ -256,6 +323,18 @@ int network_element_basis(const kt_network *net, double *Vr, int *ns, int *rank)
 // cells of the largest counts first.  Returns a cudaError_t value.
 constexpr int kSchedBuckets = 128;
 int launch_schedule(const int *count, long long ncells, unsigned *work, int *order, void *stream);
+
+// Programs of the kernels with G lanes per cell (kt_coop_tables.cu); false if the network
+// is not one they handle.  `in` / `out`: species of each reaction, -1 beyond nin / nout.
+bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *nout, const int (*in)[kMaxSide],
+                 const int (*out)[kMaxSide], const double *dH, int fp32, int G, CoopTab *tab,
+                 std::vector<unsigned char> *bytes);
+// Lanes per cell for this call (0: one cell per lane).
+int coop_group(const LaunchArgs &a, const LaunchCfg &c);
+// Whether a warp's cells fit in a block's shared memory beside the programs.
+bool coop_fits(const LaunchArgs &a, const LaunchCfg &c);
+// Several lanes per cell; returns a cudaError_t value.
+int launch_coop(const LaunchArgs &a, const LaunchCfg &c, void *stream);
 
 // Lane-per-cell kernels (N <= kLaneMaxN); returns a cudaError_t value.
 int launch_lane(const LaunchArgs &a, const LaunchCfg &c, void *stream);
