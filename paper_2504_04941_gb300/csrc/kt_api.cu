@@ -335,6 +335,9 @@ void build_blob(kt_network *n)
     }
     rp[n->ns] = static_cast<int>(re.size());
     v.nent = static_cast<int>(re.size());
+    v.nin_max = 1;
+    for (int r = 0; r < n->nr; ++r)
+        if (n->nin[r] > v.nin_max) v.nin_max = n->nin[r];
     v.shape = n->nr > 0 ? 22 : 0;
     for (int r = 0; r < n->nr; ++r)
         if (n->nin[r] != 2 || n->nout[r] != 2) v.shape = 0;
@@ -724,6 +727,7 @@ int kt::prepare_launch(const kt_network *net, int64_t ncells, const double *y_in
     a->status = status;
     a->nsub = n_substeps;
     a->nnew = n_newton;
+    a->persistent = opts->persistent != 0;
     *c = kt::LaunchCfg{opts->form, opts->persistent, opts->block_warps, opts->blocks_per_sm, cpw, opts->lane_variant};
     *host_blob = net->blob.data();
     return KT_OK;

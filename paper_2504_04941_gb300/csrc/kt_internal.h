@@ -50,6 +50,7 @@ struct NetView {
                                           // species' absorption (sum over its photo reactions)
     int ntab, tab_nT, tab_nR, off_tab;    // tables: double[ntab][nR][nT] ln k after the staged
                                           // part (global memory)
+    int nin_max;                          // largest number of reactants of a reaction
     int bytes;                            // staged part (shared memory), multiple of 16
     int bytes_warp;                       // the prefix the warp-per-cell kernels stage
                                           // (no reaction heats; photo and table
@@ -251,46 +252,44 @@ inline CoopLayout coop_layout(int N, int nr, int energy, int fp32, int blob_byte
     return L;
 }
 
-// Shared-memory layout of one warp of the warp-per-cell kernels (one cell per warp).
-// Matrices are row-major with an odd row stride NP (conflict-free column reads).
+// Shared memory of one team (one cell) of the larger-network kernels (kt_warp.cuh).
+// Matrices are column-major; the column stride LD is an odd number of 16-byte units, so the
+// 16-byte accesses of eight neighbouring columns fall into different banks.
 struct WarpLayout {
-    int NP;
-    int off_M, off_J, off_V, off_P, off_G;   // matrix, fp32 Jacobian, scales, pivots, gather
-    int off_Y, off_YF, off_YH, off_Y2, off_W;
-    int off_F0;                              // TR-BDF2: f at the step's start state
-    int off_K, off_DK;                       // rate coefficients and dk/dT (or the rates) per reaction
-    int warp_bytes, base;
+    int LD;
+    int off_M, off_J, off_V, off_G;          // matrix, Jacobian, inverse pivots, row order
+    int off_X, off_Y, off_W;                 // right-hand side, iterate, f
+    int off_RW, off_K, off_D;                // per reaction: rate, coefficient, partials
+    int off_CV, off_C;                       // C_V(T) coefficients; team exchange words
+    int warp_bytes, base;                    // bytes per team; offset of team 0
 };
 
-// share_jm (FP32 form under TR-BDF2): the FP32 Jacobian is assembled in the storage of
-// the iteration matrix and turned into I - d h J in place, since TR-BDF2 factorises
-// once per step attempt from a freshly assembled Jacobian and never re-uses it.
-inline WarpLayout warp_layout(int N, int nr, int energy, int fp32, int blob_bytes, bool share_jm = false)
+// share_jm (FP64 form; FP32 form under TR-BDF2): the Jacobian is assembled in the storage of
+// the iteration matrix and turned into I - h J in place; otherwise (FP32 form under backward
+// Euler) it is kept, since one Jacobian serves the factors for h and for h/2.
+// slim: no partials per reaction (off_D = -1; the rows of J form them from the coefficient
+// and its derivative), for networks whose partials do not fit in shared memory.
+inline WarpLayout warp_layout(int N, int nr, int energy, int fp32, int blob_bytes, bool share_jm = false,
+                              int nin_max = 2, int cvpoly = 1, bool slim = false)
 {
     WarpLayout L{};
-    L.NP = N | 1;
-    const int NN = N * L.NP;
+    const int r = fp32 ? 4 : 8, vw = 16 / r;
+    L.LD = vw * (((N + vw - 1) / vw) | (slim ? 0 : 1));
+    const int NN = N * L.LD;
     int o = 0;
-    auto take = [&](int bytes) { int r = o; o = (o + bytes + 15) & ~15; return r; };
-    if (fp32) {
-        L.off_J = take(NN * 4);
-        L.off_M = share_jm ? L.off_J : take(NN * 4);
-        L.off_V = take(N * 4);
-    } else {
-        L.off_J = -1;
-        L.off_M = take(NN * 8);
-        L.off_V = take(N * 8);
-    }
-    L.off_P = take(N * 4);
+    auto take = [&](int bytes) { int at = o; o = (o + bytes + 15) & ~15; return at; };
+    L.off_J = take(NN * r);
+    L.off_M = share_jm || !fp32 ? L.off_J : take(NN * r);
+    L.off_V = take(N * r);
     L.off_G = take(N * 4);
+    L.off_X = take(L.LD * r);
     L.off_Y = take(N * 8);
-    L.off_YF = take(N * 8);
-    L.off_YH = take(N * 8);
-    L.off_Y2 = take(N * 8);
     L.off_W = take(N * 8);
-    L.off_F0 = take(N * 8);
-    L.off_K = take(nr * 8);
-    L.off_DK = take(nr * 8);   // dk/dT; in iterations without a Jacobian, the reaction rates
+    L.off_RW = take(nr * 8);
+    L.off_K = energy && !slim ? 0 : take(nr * 8);
+    L.off_D = slim ? -1 : take(nr * r * (nin_max + (energy ? 1 : 0)));
+    L.off_CV = cvpoly ? take(10 * 8) : 0;
+    L.off_C = N > 32 ? take(2 * 3 * 4 * 4) : 0;
     L.warp_bytes = (o + 127) & ~127;
     L.base = (blob_bytes + 16 + 127) & ~127;
     return L;
@@ -338,7 +337,7 @@ int launch_coop(const LaunchArgs &a, const LaunchCfg &c, void *stream);
 
 // Lane-per-cell kernels (N <= kLaneMaxN); returns a cudaError_t value.
 int launch_lane(const LaunchArgs &a, const LaunchCfg &c, void *stream);
-// Warp-per-cell kernels (N <= kWarpMaxN); returns a cudaError_t value.
+// Larger-network kernels (N <= kWarpMaxN); returns a cudaError_t value.
 int launch_warp(const LaunchArgs &a, const LaunchCfg &c, void *stream);
 
 }  // namespace kt

@@ -1,4 +1,4 @@
-// kt_warp.cu -- launch dispatch of the warp-per-cell kernels (kt_warp.cuh) and their
+// kt_warp.cu -- launch dispatch of the larger-network kernels (kt_warp.cuh) and their
 // FP64-matrix instantiations; the FP32-LU ones are compiled in kt_warp_f32.cu.
 #include "kt_warp.cuh"
 

@@ -1,27 +1,37 @@
-// kt_warp.cuh -- warp-per-cell fused integrator for larger networks (N <= 96 unknowns).
+// kt_warp.cuh -- one to four warps per cell, for larger networks (N <= 96 unknowns).
 //
-// One warp owns one cell (the paper's Sec. 2.3 gives a whole thread block to a cell;
-// a warp keeps every exchange on shuffles and __syncwarp).  Inside the warp:
-//   rates          lanes over reactions (modified Arrhenius, Sec. 2.2.1);
-//   f and J rows   lanes over species rows, each walking its own list of
-//                  (reaction, net coefficient) pairs, so every row is accumulated
-//                  by one lane in a fixed order: deterministic, no atomics
-//                  (mass-action and thermal-coupling partials, Eq. method-jacobian);
-//   T row          lanes over columns: J_T,m = -sum_s h_s J_s,m / C_V;
-//   LU             right-looking elimination with the implicit-scaled row pivoting of
-//                  Algorithm lu-decomp: shuffle argmax for the pivot (ties to the
-//                  smaller row), lanes over columns for the row swap and the
-//                  trailing update (same factors as Crout's ordering, other rounding);
-//   solve          the right-hand side lives in registers, 3 rows per lane, and each
-//                  substitution step broadcasts the finished entry with a shuffle.
-// The sub-step control (step doubling, Newton, retry / revert, projection) is the
-// same sequence as the FP64 oracle, run warp-uniformly.
+// What bounds it: every FP64 instruction of a warp holds its scheduler's pipe for 64 cycles,
+// and a launch lasts at least as long as its longest cell, so what counts is the number of
+// FP64 instructions in one Newton iteration of one cell.  A team of NW warps owns a cell
+// (the paper's Sec. 2.3 gives it a thread block): with four, each on a scheduler of its own,
+// four FP64 pipes work on the cell.  Inside the team:
+//   rates          threads over reactions (modified Arrhenius, Sec. 2.2.1): the rate w_r and,
+//                  when a Jacobian is wanted, its partial derivatives, each formed once in
+//                  FP64 and rounded once (the rows below only add them);
+//   f and J rows   threads over species rows, each walking its own list of (reaction, +-1)
+//                  entries, so every row is accumulated by one thread in a fixed order:
+//                  deterministic, no atomics (Eq. method-jacobian);
+//   T row          threads over columns: J_T,m = -sum_s h_s J_s,m / C_V, and I - h J of the
+//                  column in the same pass;
+//   LU             right-looking with the implicit-scaled row pivoting of Algorithm
+//                  lu-decomp (same factors as Crout's ordering, other rounding) on a
+//                  column-major matrix: every warp finds the pivot by itself (integer
+//                  reductions on the bit patterns, ties to the smaller row), threads over
+//                  columns exchange the rows and update 16 bytes at a time; two team
+//                  barriers per step;
+//   solve          warp 0, the right-hand side in registers, NQ rows per lane, each finished
+//                  entry broadcast by a shuffle.
+// Sums over species go through the same 32 partial sums and shuffle tree whatever the team's
+// size, so every team size gives the same bits.  The sub-step control (step doubling or
+// TR-BDF2, Newton, retry / revert, projection) is the same sequence as the FP64 oracle, run
+// team-uniformly.
 #pragma once
 
 #include <cuda_runtime.h>
 
 #include <cmath>
 #include <cstdint>
+#include <type_traits>
 
 #include "kt_exp.cuh"
 #include "kt_internal.h"
@@ -32,8 +42,6 @@ namespace kt {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kMaxWarps = 8;
-constexpr int kQ = 3;   // rows per lane (N <= 96)
 
 struct NetS {
     const double *A, *b, *th, *h, *cv, *cnt, *ex;
@@ -46,8 +54,6 @@ __device__ __forceinline__ double wsum(double v)
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
     return __shfl_sync(kFull, v, 0);
 }
-
-__device__ __forceinline__ bool wall(bool p) { return __all_sync(kFull, p) != 0; }
 
 // x < -700 decided on the bit pattern (integer compare; same result as the FP64 compare
 // for every non-NaN x): negative and |x| > 700.0 (0x4085E00000000000).
@@ -130,129 +136,84 @@ __device__ __forceinline__ void table_rate(const NetView &nv, const double *tab,
     dk = k * ((b - a) / nv.tab_dlt) / T;
 }
 
-template <typename T>
-__device__ __forceinline__ T bcast(const T (&x)[kQ], int j)
+// Barrier of one team: T threads on the named barrier `id`.
+template <int T>
+__device__ __forceinline__ void team_sync(int id)
 {
-    const int slot = j >> 5;
-    const T v = slot == 0 ? x[0] : (slot == 1 ? x[1] : x[2]);
-    return __shfl_sync(kFull, v, j & 31);
+    if constexpr (T == 32) __syncwarp();
+    else asm volatile("barrier.sync %0, %1;" ::"r"(id), "n"(T) : "memory");
 }
 
-// Right-looking LU with implicit-scaled partial pivoting on the row-major matrix M
-// (row stride NP).  V: inverse row maxima, replaced by the inverse pivots; P: pivot
-// rows; G: composed gather index for the right-hand side.  Warp-uniform result.
-template <typename T>
-__device__ bool warp_lu(T *M, T *V, int *P, int *G, int N, int NP, int lane)
+// float -> double on the integer pipes (exact for normal values and zeros); subnormals,
+// infinities and NaNs take the conversion instruction, which occupies the FP64 pipe.
+__device__ __forceinline__ double widen(float f)
 {
-    bool ok = true;
-    for (int i = lane; i < N; i += 32) {
-        T big = T(0);
-        for (int m = 0; m < N; ++m) {
-            const T a = fabs(M[i * NP + m]);
-            big = a > big ? a : big;
-        }
-        ok = ok && big > T(0);
-        V[i] = big > T(0) ? T(1) / big : T(1);
-    }
-    ok = wall(ok);
-    __syncwarp();
-    for (int j = 0; j < N; ++j) {
-        // pivot: argmax_{i >= j} |a_ij| / rowmax_i, ties to the smaller i
-        T best = T(-1);
-        int bi = N;
-        for (int i = j + lane; i < N; i += 32) {
-            T tt = fabs(M[i * NP + j]) * V[i];
-            if (!(tt == tt)) tt = T(-1);
-            if (tt > best) {
-                best = tt;
-                bi = i;
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            const T ob = __shfl_xor_sync(kFull, best, o);
-            const int oi = __shfl_xor_sync(kFull, bi, o);
-            if (ob > best || (ob == best && oi < bi)) {
-                best = ob;
-                bi = oi;
-            }
-        }
-        best = __shfl_sync(kFull, best, 0);
-        const int p = __shfl_sync(kFull, bi, 0);
-        if (!(best > T(0)) || p >= N) return false;
-        if (p != j) {
-            for (int k = lane; k < N; k += 32) {
-                const T a = M[j * NP + k];
-                M[j * NP + k] = M[p * NP + k];
-                M[p * NP + k] = a;
-            }
-        }
-        __syncwarp();
-        if (lane == 0) {
-            const T v = V[j];
-            V[j] = V[p];
-            V[p] = v;
-            P[j] = p;
-        }
-        const T rinv = T(1) / M[j * NP + j];
-        for (int i = j + 1 + lane; i < N; i += 32) M[i * NP + j] *= rinv;
-        __syncwarp();
-        for (int k = j + 1 + lane; k < N; k += 32) {
-            const T u = M[j * NP + k];
-            for (int i = j + 1; i < N; ++i) M[i * NP + k] -= M[i * NP + j] * u;
-        }
-        __syncwarp();
-        if (lane == 0) V[j] = rinv;
-    }
-    if (lane == 0) {
-        for (int i = 0; i < N; ++i) G[i] = i;
-        for (int i = 0; i < N; ++i) {
-            const int q = P[i];
-            const int g = G[i];
-            G[i] = G[q];
-            G[q] = g;
-        }
-    }
-    __syncwarp();
-    return ok;
+    const unsigned u = __float_as_uint(f), m = u & 0x7fffffffu;
+    if (m - 0x00800000u < 0x7f000000u || m == 0u)
+        return __hiloint2double(static_cast<int>((u & 0x80000000u) | (m ? (m >> 3) + 0x38000000u : 0u)),
+                                static_cast<int>(u << 29));
+    return static_cast<double>(f);
 }
 
-// x <- M^-1 b for the factors of warp_lu; b gathered from Wb (smem) by G.
-template <typename T, typename TB>
-__device__ void warp_solve(const T *M, const T *V, const int *G, const TB *Wb, T (&x)[kQ], int N, int NP,
-                           int lane)
+__device__ __forceinline__ float fma_t(float a, float b, float c) { return fmaf(a, b, c); }
+__device__ __forceinline__ double fma_t(double a, double b, double c) { return fma(a, b, c); }
+
+// Pivot of column j: argmax_{i >= j} |M_ij| V_i over the warp's candidates c[q] (row
+// lane + 32 q, NaN already 0), ties to the smaller row; -1 if none is positive.
+template <int NQW>
+__device__ __forceinline__ int pivot_row(const float (&c)[NQW], int lane)
 {
+    unsigned k = 0;
 #pragma unroll
-    for (int q = 0; q < kQ; ++q) {
-        const int i = lane + 32 * q;
-        x[q] = i < N ? static_cast<T>(Wb[G[i]]) : T(0);
-    }
-    for (int j = 0; j < N - 1; ++j) {
-        const T xj = bcast(x, j);
+    for (int q = 0; q < NQW; ++q) k = max(k, __float_as_uint(c[q]));
+    const unsigned best = __reduce_max_sync(kFull, k);
+    unsigned row = 0xffffu;
 #pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const int i = lane + 32 * q;
-            if (i > j && i < N) x[q] -= M[i * NP + j] * xj;
-        }
-    }
-    for (int j = N - 1; j >= 0; --j) {
-        const T xj = bcast(x, j) * V[j];
-        if ((j & 31) == lane) {
-            const int slot = j >> 5;
-            if (slot == 0) x[0] = xj;
-            else if (slot == 1) x[1] = xj;
-            else x[2] = xj;
-        }
-#pragma unroll
-        for (int q = 0; q < kQ; ++q) {
-            const int i = lane + 32 * q;
-            if (i < j) x[q] -= M[i * NP + j] * xj;
-        }
-    }
+    for (int q = NQW - 1; q >= 0; --q)
+        if (__float_as_uint(c[q]) == best) row = static_cast<unsigned>(lane + 32 * q);
+    row = __reduce_min_sync(kFull, row);
+    return best == 0u ? -1 : static_cast<int>(row);
 }
 
-template <bool ENERGY, bool F32, bool PERSIST>
-__global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArgs a, const WarpLayout L)
+template <int NQW>
+__device__ __forceinline__ int pivot_row(const double (&c)[NQW], int lane)
 {
+    unsigned hi = 0;
+#pragma unroll
+    for (int q = 0; q < NQW; ++q) hi = max(hi, static_cast<unsigned>(__double2hiint(c[q])));
+    const unsigned bh = __reduce_max_sync(kFull, hi);
+    unsigned lo = 0;
+#pragma unroll
+    for (int q = 0; q < NQW; ++q)
+        if (static_cast<unsigned>(__double2hiint(c[q])) == bh)
+            lo = max(lo, static_cast<unsigned>(__double2loint(c[q])));
+    const unsigned bl = __reduce_max_sync(kFull, lo);
+    unsigned row = 0xffffu;
+#pragma unroll
+    for (int q = NQW - 1; q >= 0; --q)
+        if (static_cast<unsigned>(__double2hiint(c[q])) == bh && static_cast<unsigned>(__double2loint(c[q])) == bl)
+            row = static_cast<unsigned>(lane + 32 * q);
+    row = __reduce_min_sync(kFull, row);
+    return (bh | bl) == 0u ? -1 : static_cast<int>(row);
+}
+
+// NW warps per cell, NQ components per thread (thread t owns t, t + 32 NW, ...), NQW rows
+// per lane of one warp (N <= 32 NQW).
+template <int NW, int NQ, int NQW, bool ENERGY, bool F32>
+__global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_kernel(const LaunchArgs a, const WarpLayout L)
+{
+    using R = typename std::conditional<F32, float, double>::type;
+    constexpr int T = 32 * NW, VW = 16 / sizeof(R);
+    union Vec {   // 16 bytes of a column
+        typename std::conditional<F32, float4, double2>::type q;
+        R v[VW];
+    };
+    auto ld16 = [](const R *p) {
+        Vec x;
+        x.q = *reinterpret_cast<const decltype(x.q) *>(p);
+        return x;
+    };
+    auto st16 = [](R *p, const Vec &x) { *reinterpret_cast<decltype(Vec::q) *>(p) = x.q; };
     extern __shared__ __align__(16) unsigned char sm[];
     const NetView nv = a.nv;
     if (!stage_table(sm, a.blob, static_cast<unsigned>(nv.bytes_warp),
@@ -270,26 +231,22 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
     t.re = reinterpret_cast<const int *>(sm + nv.off_re);
     t.ex = reinterpret_cast<const double *>(sm + nv.off_exp);
     const DevOpts o = a.o;
-    const int N = nv.N, ns = nv.ns, ne = nv.ne, nr = nv.nr, NP = L.NP;
+    const int N = nv.N, ns = nv.ns, ne = nv.ne, nr = nv.nr, LD = L.LD;
     const long long nc = a.ncells;
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    unsigned char *wb = sm + L.base + wid * L.warp_bytes;
-    double *M64 = F32 ? nullptr : reinterpret_cast<double *>(wb + L.off_M);
-    double *V64 = F32 ? nullptr : reinterpret_cast<double *>(wb + L.off_V);
-    float *J32 = F32 ? reinterpret_cast<float *>(wb + L.off_J) : nullptr;
-    float *M32 = F32 ? reinterpret_cast<float *>(wb + L.off_M) : nullptr;
-    float *V32 = F32 ? reinterpret_cast<float *>(wb + L.off_V) : nullptr;
-    int *P = reinterpret_cast<int *>(wb + L.off_P);
-    int *G = reinterpret_cast<int *>(wb + L.off_G);
-    double *Y = reinterpret_cast<double *>(wb + L.off_Y);
-    double *YF = reinterpret_cast<double *>(wb + L.off_YF);
-    double *YH = reinterpret_cast<double *>(wb + L.off_YH);
-    double *Y2 = reinterpret_cast<double *>(wb + L.off_Y2);
-    double *W = reinterpret_cast<double *>(wb + L.off_W);
-    double *F0 = reinterpret_cast<double *>(wb + L.off_F0);
-    double *K = reinterpret_cast<double *>(wb + L.off_K);
-    double *DK = reinterpret_cast<double *>(wb + L.off_DK);
-    double *RW = DK;   // the reaction rates of an iteration without a Jacobian (DK is not needed then)
+    const int lane = threadIdx.x & 31, team = threadIdx.x / T, tid = threadIdx.x % T, wrp = tid >> 5;
+    auto sync = [&]() { team_sync<T>(1 + team); };
+    unsigned char *wb = sm + L.base + team * L.warp_bytes;
+    R *J = reinterpret_cast<R *>(wb + L.off_J);     // Jacobian; in M's storage when not kept apart
+    R *M = reinterpret_cast<R *>(wb + L.off_M);     // iteration matrix, then its factors
+    R *V = reinterpret_cast<R *>(wb + L.off_V);     // inverse pivots
+    R *LC = reinterpret_cast<R *>(wb + L.off_X);    // right-hand side; FP64 elimination column
+    R *D = reinterpret_cast<R *>(wb + L.off_D);     // partial derivatives [kind][reaction]
+    int *G = reinterpret_cast<int *>(wb + L.off_G); // row order of the factors
+    double *ys = reinterpret_cast<double *>(wb + L.off_Y);    // current iterate
+    double *fs = reinterpret_cast<double *>(wb + L.off_W);    // f; error terms; state being finished
+    double *ws = reinterpret_cast<double *>(wb + L.off_RW);   // reaction rates
+    double *K = reinterpret_cast<double *>(wb + L.off_K);     // rate coefficients (isothermal)
+    float *mon = reinterpret_cast<float *>(wb + L.off_C);     // per-warp convergence monitors, 2 sets
 
     long long cell = 0;
     double T_iso = 0.0, invCV = 0.0, atol_s = 0.0, dtc = a.dt;
@@ -297,7 +254,7 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
     // (five below t_mid, five from t_mid), and C_V'/C_V at the current iterate
     const bool CVP = ENERGY && nv.cvpoly != 0;
     const double *cvp = reinterpret_cast<const double *>(sm + nv.off_cvp);
-    double cvc[10];
+    double *cvc = reinterpret_cast<double *>(wb + L.off_CV);
     double dcvr = 0.0;
     // tabulated and photo rates: rate types, the cell's density weight in the tables,
     // its photo flux factor and path length, and phi'(tau) at the current iterate
@@ -307,10 +264,12 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
     const double *tabs = reinterpret_cast<const double *>(a.blob + nv.off_tab);
     int tab_iR = 0;
     double tab_w = 0.0, ph_F = 1.0, ph_dl = 0.0, ph_phi = 1.0, ph_dphi = 0.0;
+    const int nin_max = nv.nin_max, kT = nin_max;   // kinds of partials: reactants, then T
+    const bool slim = L.off_D < 0;                  // no room for partials: K and dk/dT (in ws) instead
 
     // k and dk/dT of reaction r at T (lt = ln(T/T_ref), lT = ln T); photo-reactions take
     // the current phi(tau) (dk/dT = 0)
-    auto rate = [&](int r, double T, double lt, double lT, double invT, double &k, double &dk) {
+    auto rate = [&](int r, double Tc, double lt, double lT, double invT, double &k, double &dk) {
         const int ty = nv.special ? rtype[r] : 0;
         if (ty == 0) {
             arrhenius(t, r, lt, invT, k, dk);
@@ -318,272 +277,528 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
             k = ph_F * sigr[r] * ph_phi;
             dk = 0.0;
         } else {
-            table_rate(nv, tabs, ty >> 8, tab_iR, tab_w, T, lT, k, dk);
+            table_rate(nv, tabs, ty >> 8, tab_iR, tab_w, Tc, lT, k, dk);
         }
     };
-    int nnew = 0;
+    int nnew = 0, flip = 0;
 
+    double Y[NQ], F0[NQ], YF[NQ], YH[NQ], CUR[NQ], W[NQ];   // own components
+    auto own = [&](int q) { return tid + T * q; };
     auto yin = [&](int s) { return a.y_in[static_cast<long long>(s) * nc + cell]; };
 
     auto load_pre = [&]() {
-        for (int s = lane; s < ns; s += 32) {
-            const double v = yin(s);
-            Y[s] = v > 0.0 ? v : 0.0;
-        }
         const double Tin = a.T_in[cell];
         T_iso = Tin < nv.t_min ? nv.t_min : (Tin > nv.t_max ? nv.t_max : Tin);
-        if (ENERGY && lane == 0) Y[ns] = T_iso;
-        __syncwarp();
-    };
-
-    // species rows of f (into W) and, when wantJ, of J (into the FP64 or FP32 matrix),
-    // then the temperature row; all at state yt with the coefficients in K / DK.
-    auto rows = [&](const double *yt, bool wantJ) {
-        if (!wantJ) {
-            // f alone: each reaction's rate w_r = k_r n_i n_j (n_k) once, lanes over
-            // reactions, then every species row adds +-w_r per list entry (every entry
-            // has a coefficient of +-1), the sign applied on the bit pattern: one FP64
-            // add per entry whatever the signs of the 32 rows a warp sums at once, and
-            // about a quarter of the FP64 work of forming k n_i n_j in every row a
-            // reaction appears in.
-            for (int r = lane; r < nr; r += 32) {
-                const unsigned long long ix = t.idx[r];
-                const int nin = static_cast<int>(ix & 0x7f);
-                const double y0 = yt[(ix >> 16) & 0xff];
-                const double y1 = nin > 1 ? yt[(ix >> 24) & 0xff] : 1.0;
-                const double y2 = nin > 2 ? yt[(ix >> 32) & 0xff] : 1.0;
-                RW[r] = K[r] * (y0 * y1) * y2;
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int i = own(q);
+            Y[q] = 0.0;
+            if (i < ns) {
+                const double v = yin(i);
+                Y[q] = v > 0.0 ? v : 0.0;
+            } else if (ENERGY && i == ns) {
+                Y[q] = T_iso;
             }
-            __syncwarp();
-            for (int s = lane; s < ns; s += 32) {
-                double f = 0.0;
-                const int e1 = t.rp[s + 1];
-                for (int e = t.rp[s]; e < e1; ++e) {
-                    const int ent = t.re[e];
-                    // -1 is stored as 0xff: its bit 7 becomes the sign bit of w_r
-                    const long long sign = static_cast<long long>(ent & 0x80) << 56;
-                    f += __longlong_as_double(__double_as_longlong(RW[ent >> 8]) ^ sign);
-                }
-                W[s] = f;
-            }
-        }
-        for (int s = lane; wantJ && s < ns; s += 32) {
-            double f = 0.0;
-            if (wantJ) {
-                if (F32) {
-                    for (int m = 0; m < N; ++m) J32[s * NP + m] = 0.0f;
-                } else {
-                    for (int m = 0; m < N; ++m) M64[s * NP + m] = 0.0;
-                }
-            }
-            const int e1 = t.rp[s + 1];
-            double gph = 0.0;    // photo: sum over the row's photo reactions of nu F sigma_r n_i phi' dl
-            for (int e = t.rp[s]; e < e1; ++e) {
-                const int ent = t.re[e];
-                const int r = ent >> 8;
-                const double nu = static_cast<double>(static_cast<signed char>(ent & 0xff));
-                const unsigned long long ix = t.idx[r];
-                const int nin = static_cast<int>(ix & 0x7f);
-                const int i0 = static_cast<int>((ix >> 16) & 0xff), i1 = static_cast<int>((ix >> 24) & 0xff),
-                          i2 = static_cast<int>((ix >> 32) & 0xff);
-                const double k = K[r];
-                const double y0 = yt[i0];
-                const double y1 = nin > 1 ? yt[i1] : 1.0;
-                const double y2 = nin > 2 ? yt[i2] : 1.0;
-                const double p01 = y0 * y1;
-                f += nu * (k * p01 * y2);
-                if (wantJ && nv.nphoto && rtype[r] == 2) gph += nu * (ph_F * sigr[r] * y0 * ph_dphi * ph_dl);
-                if (wantJ) {
-                    // two different reactants: the row entries i0, i1 (and T) differ, so
-                    // they are loaded first and stored after (one shared-memory round trip
-                    // instead of a chain of read-modify-writes); same updates either way
-                    const bool two = nin == 2 && i0 != i1;
-                    if (F32) {
-                        float *row = J32 + s * NP;
-                        if (two) {
-                            const float a0 = row[i0], a1 = row[i1], aT = ENERGY ? row[ns] : 0.0f;
-                            row[i0] = a0 + static_cast<float>(nu * (k * y1 * y2));
-                            row[i1] = a1 + static_cast<float>(nu * (k * y0 * y2));
-                            if (ENERGY) row[ns] = aT + static_cast<float>(nu * (DK[r] * p01 * y2));
-                        } else {
-                            row[i0] += static_cast<float>(nu * (k * y1 * y2));
-                            if (nin > 1) row[i1] += static_cast<float>(nu * (k * y0 * y2));
-                            if (nin > 2) row[i2] += static_cast<float>(nu * (k * p01));
-                            if (ENERGY) row[ns] += static_cast<float>(nu * (DK[r] * p01 * y2));
-                        }
-                    } else {
-                        double *row = M64 + s * NP;
-                        if (two) {
-                            const double a0 = row[i0], a1 = row[i1], aT = ENERGY ? row[ns] : 0.0;
-                            row[i0] = a0 + nu * (k * y1 * y2);
-                            row[i1] = a1 + nu * (k * y0 * y2);
-                            if (ENERGY) row[ns] = aT + nu * (DK[r] * p01 * y2);
-                        } else {
-                            row[i0] += nu * (k * y1 * y2);
-                            if (nin > 1) row[i1] += nu * (k * y0 * y2);
-                            if (nin > 2) row[i2] += nu * (k * p01);
-                            if (ENERGY) row[ns] += nu * (DK[r] * p01 * y2);
-                        }
-                    }
-                }
-            }
-            // dw/dn_m of a photo rate through tau: + (sum) sigma_m for every absorber m
-            if (wantJ && gph != 0.0) {
-                for (int m = 0; m < ns; ++m) {
-                    if (F32) J32[s * NP + m] += static_cast<float>(gph * sigs[m]);
-                    else M64[s * NP + m] += gph * sigs[m];
-                }
-            }
-            W[s] = f;
-        }
-        __syncwarp();
-        if (ENERGY) {
-            double q = 0.0;
-            for (int s = lane; s < ns; s += 32) q += t.h[s] * W[s];
-            q = wsum(q);
-            if (wantJ) {
-                for (int m = lane; m < N; m += 32) {
-                    double c = 0.0;
-                    if (F32) {
-                        for (int s = 0; s < ns; ++s) c += t.h[s] * static_cast<double>(J32[s * NP + m]);
-                        J32[ns * NP + m] = static_cast<float>(-c * invCV);
-                    } else {
-                        for (int s = 0; s < ns; ++s) c += t.h[s] * M64[s * NP + m];
-                        M64[ns * NP + m] = -c * invCV;
-                    }
-                }
-            }
-            __syncwarp();
-            if (lane == 0) {
-                W[ns] = -q * invCV;
-                // d f_T / d T of C_V(T): -f_T C_V'/C_V
-                if (CVP && wantJ) {
-                    if (F32) J32[ns * NP + ns] -= static_cast<float>(W[ns] * dcvr);
-                    else M64[ns * NP + ns] -= W[ns] * dcvr;
-                }
-            }
-            __syncwarp();
         }
     };
 
-    auto coefficients = [&](double T, const double *yt) {
+    auto put = [&](double *to, const double (&v)[NQ]) {
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            if (own(q) < N) to[own(q)] = v[q];
+    };
+
+    // Rates at the state in ys (written and synchronised by the caller): w_r into ws and,
+    // when wantJ, the partials into D; then the species rows of f into fs / W and, when
+    // wantJ, of J; the temperature row of f.  hph is only read when the iteration matrix
+    // replaces J in place (L.off_J == L.off_M with fuse).
+    auto rates_rows = [&](bool wantJ) {
+        const double Tc = ENERGY ? ys[ns] : T_iso;
         if (nv.nphoto) {
             // optical depth tau = dl sum_s n_s sigma_s of the iterate, then phi(tau)
             double sg = 0.0;
-            for (int s = lane; s < ns; s += 32) sg += yt[s] * sigs[s];
+            for (int s = lane; s < ns; s += 32) sg = fma(ys[s], sigs[s], sg);
             photo_phi(ph_dl * wsum(sg), ph_phi, ph_dphi);
-            if (!ENERGY) {
-                for (int r = lane; r < nr; r += 32)
-                    if (rtype[r] == 2) K[r] = ph_F * sigr[r] * ph_phi;
-                __syncwarp();
-            }
         }
         if (CVP) {
-            const int o5 = T < nv.t_mid ? 0 : 5;
-            const double cv = (((cvc[o5 + 4] * T + cvc[o5 + 3]) * T + cvc[o5 + 2]) * T + cvc[o5 + 1]) * T + cvc[o5];
-            const double dcv = ((4.0 * cvc[o5 + 4] * T + 3.0 * cvc[o5 + 3]) * T + 2.0 * cvc[o5 + 2]) * T + cvc[o5 + 1];
+            const int o5 = Tc < nv.t_mid ? 0 : 5;
+            const double cv = (((cvc[o5 + 4] * Tc + cvc[o5 + 3]) * Tc + cvc[o5 + 2]) * Tc + cvc[o5 + 1]) * Tc + cvc[o5];
+            const double dcv = ((4.0 * cvc[o5 + 4] * Tc + 3.0 * cvc[o5 + 3]) * Tc + 2.0 * cvc[o5 + 2]) * Tc + cvc[o5 + 1];
             invCV = 1.0 / cv;
             dcvr = dcv * invCV;
         }
+        double lt = 0.0, invT = 0.0, lT = 0.0;
         if (ENERGY) {
-            const double lt = log_t(T, nv.t_ref), invT = 1.0 / T;
-            const double lT = nv.ntab ? log(T) : 0.0;
-            for (int r = lane; r < nr; r += 32) {
-                double k, dk;
-                rate(r, T, lt, lT, invT, k, dk);
-                K[r] = k;
-                DK[r] = dk;
+            lt = log_t(Tc, nv.t_ref);
+            invT = 1.0 / Tc;
+            lT = nv.ntab ? log(Tc) : 0.0;
+        }
+        for (int r = tid; r < nr; r += T) {
+            double k, dk = 0.0;
+            if (ENERGY) rate(r, Tc, lt, lT, invT, k, dk);
+            else k = nv.nphoto && rtype[r] == 2 ? ph_F * sigr[r] * ph_phi : K[r];
+            const unsigned long long ix = t.idx[r];
+            const int nin = static_cast<int>(ix & 0x7f);
+            const double y0 = ys[(ix >> 16) & 0xff];
+            const double y1 = nin > 1 ? ys[(ix >> 24) & 0xff] : 1.0;
+            const double p01 = __dmul_rn(y0, y1);
+            double w = __dmul_rn(k, p01), y2 = 1.0;
+            if (nin_max > 2) {
+                y2 = nin > 2 ? ys[(ix >> 32) & 0xff] : 1.0;
+                w = __dmul_rn(w, y2);
             }
-            __syncwarp();
+            ws[r] = w;
+            if (wantJ && slim) {
+                if (ENERGY) {
+                    K[r] = k;
+                    ws[r] = dk;
+                } else {
+                    K[r] = k;   // (a photo rate at this iterate)
+                }
+            } else if (wantJ) {
+                double d0 = __dmul_rn(k, y1), d1 = __dmul_rn(k, y0);
+                if (nin_max > 2) {
+                    d0 = __dmul_rn(d0, y2);
+                    d1 = __dmul_rn(d1, y2);
+                    D[2 * nr + r] = static_cast<R>(__dmul_rn(k, p01));
+                }
+                D[r] = static_cast<R>(d0);
+                if (nin_max > 1) D[nr + r] = static_cast<R>(d1);
+                if (ENERGY) {
+                    double dT = __dmul_rn(dk, p01);
+                    if (nin_max > 2) dT = __dmul_rn(dT, y2);
+                    D[kT * nr + r] = static_cast<R>(dT);
+                }
+            }
+        }
+        sync();
+        // f: every species row adds +-w_r per list entry (every entry has a coefficient of
+        // +-1, the sign applied on the bit pattern), the next entry's rate loaded ahead
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int s = own(q);
+            double f = 0.0;
+            if (s < ns && !(wantJ && slim)) {
+                const int e0 = t.rp[s], e1 = t.rp[s + 1];
+                int n0 = e0 < e1 ? t.re[e0] : 0, n1 = e0 + 1 < e1 ? t.re[e0 + 1] : 0;
+                double w0 = e0 < e1 ? ws[n0 >> 8] : 0.0;
+                for (int e = e0; e < e1; ++e) {
+                    const int n2 = e + 2 < e1 ? t.re[e + 2] : 0;
+                    const double w1 = ws[n1 >> 8];
+                    // -1 is stored as 0xff: its bit 7 becomes the sign bit of w_r
+                    f += __longlong_as_double(__double_as_longlong(w0) ^ (static_cast<long long>(n0 & 0x80) << 56));
+                    n0 = n1;
+                    n1 = n2;
+                    w0 = w1;
+                }
+                fs[s] = f;
+            }
+            W[q] = f;
+        }
+        if (wantJ) {
+            for (int s = tid; s < ns; s += T) {
+                R *row = J + s;   // entry m of the row at m * LD
+                for (int m = 0; m < N; ++m) row[m * LD] = R(0);
+                const int e0 = t.rp[s], e1 = t.rp[s + 1];
+                double gph = 0.0;    // photo: sum over the row's photo reactions of nu F sigma_r n_i phi' dl
+                R aT = R(0);
+                // an entry's reaction and partials are loaded while the one before it updates
+                // the row (what remains is the row's own read-modify-write chain)
+                struct Entry {
+                    int ent;
+                    unsigned long long ix;
+                    R d0, d1, dT;
+                };
+                double f = 0.0;
+                auto load = [&](int e) {
+                    Entry n{};
+                    if (e < e1) {
+                        n.ent = t.re[e];
+                        const int r = n.ent >> 8;
+                        n.ix = t.idx[r];
+                        if (slim) return n;
+                        n.d0 = D[r];
+                        if (nin_max > 1) n.d1 = D[nr + r];
+                        if (ENERGY) n.dT = D[kT * nr + r];
+                    }
+                    return n;
+                };
+                Entry n = load(e0);
+                for (int e = e0; e < e1; ++e) {
+                    Entry c = n;
+                    R d2 = R(0);
+                    n = load(e + 1);
+                    const int nin = static_cast<int>(c.ix & 0x7f);
+                    const int i0 = static_cast<int>((c.ix >> 16) & 0xff), i1 = static_cast<int>((c.ix >> 24) & 0xff);
+                    if (slim) {
+                        const int r = c.ent >> 8;
+                        const double k = K[r], y0 = ys[i0], y1 = nin > 1 ? ys[i1] : 1.0;
+                        const double y2 = nin > 2 ? ys[(c.ix >> 32) & 0xff] : 1.0, p01 = __dmul_rn(y0, y1);
+                        const double w = __dmul_rn(__dmul_rn(k, p01), y2);
+                        f += (c.ent & 0x80) ? -w : w;
+                        c.d0 = static_cast<R>(__dmul_rn(__dmul_rn(k, y1), y2));
+                        c.d1 = static_cast<R>(__dmul_rn(__dmul_rn(k, y0), y2));
+                        d2 = static_cast<R>(__dmul_rn(k, p01));
+                        if (ENERGY) c.dT = static_cast<R>(__dmul_rn(__dmul_rn(ws[r], p01), y2));
+                    } else if (nin > 2) {
+                        d2 = D[2 * nr + (c.ent >> 8)];
+                    }
+                    const R sg = (c.ent & 0x80) ? R(-1) : R(1);   // fma(+-1, d, a) = a +- d
+                    if (nin == 2 && i0 != i1) {
+                        // the two entries differ: both loaded, then both stored
+                        const R a0 = row[i0 * LD], a1 = row[i1 * LD];
+                        row[i0 * LD] = fma_t(sg, c.d0, a0);
+                        row[i1 * LD] = fma_t(sg, c.d1, a1);
+                    } else {
+                        const int i2 = static_cast<int>((c.ix >> 32) & 0xff);
+                        row[i0 * LD] = fma_t(sg, c.d0, row[i0 * LD]);
+                        if (nin > 1) row[i1 * LD] = fma_t(sg, c.d1, row[i1 * LD]);
+                        if (nin > 2) row[i2 * LD] = fma_t(sg, d2, row[i2 * LD]);
+                    }
+                    if (ENERGY) aT = fma_t(sg, c.dT, aT);
+                    if (nv.nphoto && rtype[c.ent >> 8] == 2) {
+                        const double g = ph_F * sigr[c.ent >> 8] * ys[i0] * ph_dphi * ph_dl;
+                        gph += (c.ent & 0x80) ? -g : g;
+                    }
+                }
+                if (ENERGY) row[ns * LD] = aT;
+                if (slim) {
+                    fs[s] = f;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+                        if (own(q) == s) W[q] = f;
+                }
+                // dw/dn_m of a photo rate through tau: + (sum) sigma_m for every absorber m
+                if (gph != 0.0)
+                    for (int m = 0; m < ns; ++m) {
+                        if constexpr (F32) row[m * LD] += static_cast<float>(__dmul_rn(gph, sigs[m]));
+                        else row[m * LD] = fma(gph, sigs[m], row[m * LD]);
+                    }
+            }
+        }
+        if (ENERGY) {
+            sync();
+            if (wrp == ((ns % T) >> 5)) {   // the warp that owns the temperature
+                double qs = 0.0;
+                for (int s = lane; s < ns; s += 32) qs = fma(t.h[s], fs[s], qs);
+                qs = wsum(qs);
+#pragma unroll
+                for (int q = 0; q < NQ; ++q)
+                    if (own(q) == ns) W[q] = -qs * invCV;
+            }
         }
     };
 
-    // factor state of the FP32 form
-    bool luok32 = false;
-    double h_fact = -1.0;
+    // temperature row of J (threads over columns) and, when hph > 0, I - hph J into M in the
+    // same pass over the column
+    auto t_row = [&](double hph) {
+        const R hr = static_cast<R>(hph);
+        sync();
+        for (int m = tid; m < N; m += T) {
+            double c = 0.0;
+            const R *jm = J + m * LD;
+            R *mm = M + m * LD;
+            int s = 0;
+            for (; s + VW <= ns; s += VW) {
+                const Vec j = ld16(jm + s);
+                Vec x;
+#pragma unroll
+                for (int e = 0; e < VW; ++e) {
+                    if (ENERGY) {
+                        if constexpr (F32) c = fma(t.h[s + e], widen(j.v[e]), c);
+                        else c = fma(t.h[s + e], j.v[e], c);
+                    }
+                    x.v[e] = fma_t(-hr, j.v[e], s + e == m ? R(1) : R(0));
+                }
+                if (hph > 0.0) st16(mm + s, x);
+            }
+            for (; s < ns; ++s) {
+                const R j = jm[s];
+                if (ENERGY) {
+                    if constexpr (F32) c = fma(t.h[s], widen(j), c);
+                    else c = fma(t.h[s], j, c);
+                }
+                if (hph > 0.0) mm[s] = fma_t(-hr, j, s == m ? R(1) : R(0));
+            }
+            if (ENERGY) {
+                R jt = static_cast<R>(-c * invCV);
+                // d f_T / d T of C_V(T): -f_T C_V'/C_V
+                if (CVP && m == ns) {
+                    if constexpr (F32) jt -= static_cast<float>(__dmul_rn(fs[ns], dcvr));
+                    else jt = fma(-fs[ns], dcvr, jt);
+                }
+                J[m * LD + ns] = jt;
+                if (hph > 0.0) mm[ns] = fma_t(-hr, jt, m == ns ? R(1) : R(0));
+            }
+        }
+    };
 
-    // One backward-Euler solve yt = yb + hph f(yt) by Newton from the guess in yt.
-    // fmode (FP32 form): 2 assemble J at the guess and factor; 1 factor from the
-    // stored J; 0 reuse the current factor.
-    auto be_solve = [&](const double *yb, double *yt, double hph, int fmode) -> bool {
+    // Right-looking LU of M; G: composed gather index of the right-hand side, V: inverse
+    // pivots.  Columns are contiguous, so a thread updates a column 16 bytes at a time
+    // (measured on 65 unknowns: 260k cycles per factorisation row-major, one value at a
+    // time).  Team-uniform result.
+    auto lu = [&]() -> bool {
+        constexpr int H = NW > 1 ? 2 : 1;   // threads per column
+        sync();
+        R v[NQW];   // inverse row maxima of rows lane + 32 q, the same in every warp
+        bool ok = true;
+#pragma unroll
+        for (int q = 0; q < NQW; ++q) {
+            const int i = lane + 32 * q;
+            v[q] = R(1);
+            if (i < N) {
+                R big = R(0);
+#pragma unroll 4
+                for (int m = 0; m < N; ++m) {
+                    const R x = fabs(M[m * LD + i]);
+                    big = x > big ? x : big;
+                }
+                ok = ok && big > R(0);
+                if (big > R(0)) v[q] = R(1) / big;
+            }
+        }
+        ok = __all_sync(kFull, ok) != 0;
+        for (int i = tid; i < N; i += T) G[i] = i;
+        for (int j = 0; j < N; ++j) {
+            sync();   // the previous step's update is complete
+            R *mj = M + j * LD;
+            R c[NQW];
+#pragma unroll
+            for (int q = 0; q < NQW; ++q) {
+                const int i = lane + 32 * q;
+                R x = R(0);
+                if (i >= j && i < N) {
+                    x = fabs(mj[i]) * v[q];
+                    if (!(x == x)) x = R(0);
+                }
+                c[q] = x;
+            }
+            const int p = pivot_row(c, lane);
+            if (p < 0) return false;
+            const R piv = mj[p], mjj = mj[j], rinv = R(1) / piv;
+            // the multipliers of the rows below, as they stand after rows j and p exchange
+            for (int i = j + 1 + tid; i < N; i += T) {
+                const R x = i == p ? mjj : mj[i];
+                LC[i] = x * rinv;
+            }
+            if (p != j) {
+                for (int k = tid; k < N; k += T)
+                    if (k != j) {
+                        R *mk = M + k * LD;
+                        const R x = mk[j];
+                        mk[j] = mk[p];
+                        mk[p] = x;
+                    }
+                // row scales follow their rows
+                R vj = R(0);
+#pragma unroll
+                for (int q = 0; q < NQW; ++q)
+                    if (j >> 5 == q) vj = v[q];
+                vj = __shfl_sync(kFull, vj, j & 31);
+#pragma unroll
+                for (int q = 0; q < NQW; ++q)
+                    if (lane + 32 * q == p) v[q] = vj;
+            }
+            if (tid == T - 1) {
+                const int g = G[j];
+                G[j] = G[p];
+                G[p] = g;
+                V[j] = rinv;
+            }
+            sync();
+            for (int i = j + tid; i < N; i += T) mj[i] = i == j ? piv : LC[i];
+            // rows j + 1 .. of the columns to the right, VW rows at a time from the chunk that
+            // holds row j + 1 (its rows up to j stay)
+            const int i0 = (j + 1) & ~(VW - 1);
+            for (int k = j + 1 + tid / H; k < N; k += T / H) {
+                R *mk = M + k * LD;
+                const R u = mk[j];
+                int i = i0 + (tid % H) * VW;
+                if (H == 1 || tid % H == 0) {
+                    const Vec l = ld16(LC + i);
+                    Vec x = ld16(mk + i);
+#pragma unroll
+                    for (int e = 0; e < VW; ++e) {
+                        const R y = fma_t(-l.v[e], u, x.v[e]);
+                        if (i + e > j) x.v[e] = y;
+                    }
+                    st16(mk + i, x);
+                    i += H * VW;
+                }
+#pragma unroll 2
+                for (; i < N; i += H * VW) {
+                    const Vec l = ld16(LC + i);
+                    Vec x = ld16(mk + i);
+#pragma unroll
+                    for (int e = 0; e < VW; ++e) x.v[e] = fma_t(-l.v[e], u, x.v[e]);
+                    st16(mk + i, x);
+                }
+            }
+        }
+        sync();
+        return ok;
+    };
+
+    // x <- M^-1 b for the factors of lu(): b gathered from LC by G, the solution left in LC.
+    // Each step is a shuffle and an update; the factors of eight steps are loaded ahead.
+    auto solve = [&]() {
+        sync();
+        if (wrp == 0) {
+            R x[NQW];
+            int at[NQW];   // row of the lane, the last row where there is none (not stored)
+#pragma unroll
+            for (int q = 0; q < NQW; ++q) {
+                const int i = lane + 32 * q;
+                at[q] = i < N ? i : N - 1;
+                x[q] = LC[G[at[q]]];
+            }
+            __syncwarp();
+#pragma unroll
+            for (int jq = 0; jq < NQW; ++jq) {
+                const int n = N - 1 - 32 * jq < 32 ? N - 1 - 32 * jq : 32;
+                auto steps = [&](int jj, auto count) {
+                    constexpr int B = decltype(count)::value;
+                    R m[B][NQW];
+#pragma unroll
+                    for (int e = 0; e < B; ++e)
+#pragma unroll
+                        for (int q = jq; q < NQW; ++q) m[e][q] = M[(32 * jq + jj + e) * LD + at[q]];
+#pragma unroll
+                    for (int e = 0; e < B; ++e) {
+                        const R xj = __shfl_sync(kFull, x[jq], jj + e);
+#pragma unroll
+                        for (int q = jq; q < NQW; ++q) {
+                            const R y = fma_t(-m[e][q], xj, x[q]);
+                            x[q] = q > jq || lane > jj + e ? y : x[q];
+                        }
+                    }
+                };
+                int jj = 0;
+                for (; jj + 8 <= n; jj += 8) steps(jj, std::integral_constant<int, 8>());
+                for (; jj < n; ++jj) steps(jj, std::integral_constant<int, 1>());
+            }
+#pragma unroll
+            for (int jq = NQW - 1; jq >= 0; --jq) {
+                const int n = N - 32 * jq < 32 ? N - 32 * jq : 32;
+                auto steps = [&](int top, auto count) {   // columns top, top - 1, ..
+                    constexpr int B = decltype(count)::value;
+                    R m[B][NQW], vi[B];
+#pragma unroll
+                    for (int e = 0; e < B; ++e) {
+                        vi[e] = V[32 * jq + top - e];
+#pragma unroll
+                        for (int q = 0; q <= jq; ++q) m[e][q] = M[(32 * jq + top - e) * LD + at[q]];
+                    }
+#pragma unroll
+                    for (int e = 0; e < B; ++e) {
+                        const R xj = __shfl_sync(kFull, x[jq], top - e) * vi[e];
+#pragma unroll
+                        for (int q = 0; q <= jq; ++q) {
+                            const R y = fma_t(-m[e][q], xj, x[q]);
+                            if (q < jq) x[q] = y;
+                            else x[q] = lane < top - e ? y : (lane == top - e ? xj : x[q]);
+                        }
+                    }
+                };
+                int top = n - 1;
+                for (; top >= 7; top -= 8) steps(top, std::integral_constant<int, 8>());
+                for (; top >= 0; --top) steps(top, std::integral_constant<int, 1>());
+            }
+#pragma unroll
+            for (int q = 0; q < NQW; ++q)
+                if (lane + 32 * q < N) LC[lane + 32 * q] = x[q];
+        }
+        sync();
+    };
+
+    bool luok = false;
+    const double natol_f = F32 ? o.newton_atol_frac * kF32NewtonAtolScale : o.newton_atol_frac;
+
+    // One solve y = b + hph f(y) by Newton from the guess in CUR (ys holds it too), b in YB.
+    // fmode (FP32 form): 2 assemble J at the guess and factor; 1 factor from the stored J;
+    // 0 reuse the current factor.
+    auto be_solve = [&](const double (&yb)[NQ], double hph, int fmode) -> bool {
         int refresh = 0;
-        bool doJ = F32 && fmode == 2, doF = F32 && fmode >= 1;
+        bool doJ = !F32 || fmode == 2, doF = !F32 || fmode >= 1;
         float dprev = 0.0f, dprevr = 0.0f;
+        const double natol = __dmul_rn(natol_f, atol_s);
         for (int it = 0;; ++it) {
             ++nnew;
-            const double T = ENERGY ? yt[ns] : T_iso;
-            if (!(T > 0.0)) return false;
-            coefficients(T, yt);
-            bool luok;
-            double x[kQ];
-            if (!F32) {
-                rows(yt, true);
-                for (int i = lane; i < N; i += 32) {
-                    double *row = M64 + i * NP;
-                    for (int m = 0; m < N; ++m) row[m] = (i == m ? 1.0 : 0.0) - hph * row[m];
-                    W[i] = -(yt[i] - yb[i] - hph * W[i]);
-                }
-                __syncwarp();
-                luok = warp_lu<double>(M64, V64, P, G, N, NP, lane);
-                if (!luok) return false;
-                warp_solve<double, double>(M64, V64, G, W, x, N, NP, lane);
-            } else {
-                rows(yt, doJ);
-                if (doF) {
-                    for (int i = lane; i < N; i += 32)
-                        for (int m = 0; m < N; ++m)
-                            M32[i * NP + m] = (i == m ? 1.0f : 0.0f) - static_cast<float>(hph) * J32[i * NP + m];
-                    __syncwarp();
-                    luok32 = warp_lu<float>(M32, V32, P, G, N, NP, lane);
-                    h_fact = hph;
-                }
-                doJ = false;
-                doF = false;
-                if (!luok32) return false;
-                for (int i = lane; i < N; i += 32) W[i] = -(yt[i] - yb[i] - hph * W[i]);
-                __syncwarp();
-                float xf[kQ];
-                warp_solve<float, double>(M32, V32, G, W, xf, N, NP, lane);
+            sync();
+            const double Tc = ENERGY ? ys[ns] : T_iso;
+            if (!(Tc > 0.0)) return false;
+            rates_rows(doJ);
+            if (CVP && doJ) {
 #pragma unroll
-                for (int q = 0; q < kQ; ++q) x[q] = static_cast<double>(xf[q]);
+                for (int q = 0; q < NQ; ++q)
+                    if (own(q) == ns) fs[ns] = W[q];
             }
+            if (doJ) t_row(doF ? hph : 0.0);
+            else if (doF) {   // a new h with the stored J
+                const R hr = static_cast<R>(hph);
+                for (int m = tid; m < N; m += T)
+                    for (int s = 0; s < N; ++s) M[m * LD + s] = fma_t(-hr, J[m * LD + s], s == m ? R(1) : R(0));
+            }
+            if (doF) luok = lu();
+            if (F32) doJ = doF = false;
+            if (!luok) return false;
+#pragma unroll
+            for (int q = 0; q < NQ; ++q)
+                if (own(q) < N)
+                    LC[own(q)] = static_cast<R>(-fma(-hph, W[q], __dadd_rn(CUR[q], -yb[q])));
+            solve();
             bool conv = true;
             // contraction monitors (FP32 is plenty): dmax = max |delta|/tol, dmaxr =
             // max |delta| / (newton_rtol |y|), the purely relative part of the tolerance
             float dmax = 0.0f, dmaxr = 0.0f;
-            const double natol = (F32 ? o.newton_atol_frac * kF32NewtonAtolScale : o.newton_atol_frac) * atol_s;
 #pragma unroll
-            for (int q = 0; q < kQ; ++q) {
-                const int i = lane + 32 * q;
+            for (int q = 0; q < NQ; ++q) {
+                const int i = own(q);
                 if (i < N) {
-                    const double y = yt[i] + x[q];
-                    yt[i] = y;
-                    const double tol = (i < ns ? natol : 0.0) + o.newton_rtol * fabs(y);
-                    if (!(fabs(x[q]) <= tol)) conv = false;
-                    if (F32) {
-                        const float ad = static_cast<float>(fabs(x[q])), tf = static_cast<float>(tol);
+                    const double x = static_cast<double>(LC[i]);
+                    const double y = __dadd_rn(CUR[q], x);
+                    CUR[q] = y;
+                    ys[i] = y;
+                    const double ny = __dmul_rn(o.newton_rtol, fabs(y));
+                    const double tol = fma(o.newton_rtol, fabs(y), i < ns ? natol : 0.0);
+                    if (!(fabs(x) <= tol)) conv = false;
+                    if constexpr (F32) {
+                        const float ad = fabsf(LC[i]), tf = static_cast<float>(tol);
                         const float r = __fdiv_rn(ad, fmaxf(tf, 1e-37f));
                         // the relative part newton_rtol |y| formed directly: as a difference
                         // tf - natol in FP32 it rounds to an ulp of natol for trace species
-                        const float trl = static_cast<float>(o.newton_rtol * fabs(y));
+                        const float trl = static_cast<float>(ny);
                         const float rr = __fdiv_rn(ad, fmaxf(trl, 1e-37f));
                         dmax = r > dmax ? r : dmax;
                         dmaxr = rr > dmaxr ? rr : dmaxr;
                     }
                 }
             }
-            __syncwarp();
-            conv = wall(conv);
+            conv = __all_sync(kFull, conv) != 0;
+            if constexpr (F32) {   // non-negative: ordered like their bit patterns
+                dmax = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(dmax)));
+                dmaxr = __uint_as_float(__reduce_max_sync(kFull, __float_as_uint(dmaxr)));
+            }
+            if constexpr (NW > 1) {
+                float *slot = mon + 3 * NW * flip;
+                flip ^= 1;
+                if (lane == 0) {
+                    slot[3 * wrp] = conv ? 1.0f : 0.0f;
+                    slot[3 * wrp + 1] = dmax;
+                    slot[3 * wrp + 2] = dmaxr;
+                }
+                sync();
+#pragma unroll
+                for (int w = 0; w < NW; ++w) {
+                    conv = conv && slot[3 * w] != 0.0f;
+                    dmax = fmaxf(dmax, slot[3 * w + 1]);
+                    dmaxr = fmaxf(dmaxr, slot[3 * w + 2]);
+                }
+            }
             if (conv) return true;
             if (!F32) {
                 if (it + 1 >= o.max_newton) return false;
             } else {
-                for (int off = 16; off > 0; off >>= 1) {
-                    dmax = fmaxf(dmax, __shfl_xor_sync(kFull, dmax, off));
-                    dmaxr = fmaxf(dmaxr, __shfl_xor_sync(kFull, dmaxr, off));
-                }
-                dmax = __shfl_sync(kFull, dmax, 0);
-                dmaxr = __shfl_sync(kFull, dmaxr, 0);
                 if (!isfinite(dmax)) return false;
                 // stop on the contraction rate (Hairer & Wanner, Solving ODEs II, Sec. IV.8):
                 // with theta = dmaxr / dprevr < 1/2 the error left after this update is about
@@ -611,9 +826,9 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
     // Sub-steps over [0, dtc] in either scheme; every Newton solve goes through the one
     // call of be_solve below (one inlined copy of the solver per kernel).
     //   backward Euler with step doubling: stage 0 the full step h from Y (-> YF),
-    //     stage 1 the first half step from Y (-> YH), stage 2 the second from YH (-> Y2)
+    //     stage 1 the first half step from Y (-> YH), stage 2 the second from YH
     //   TR-BDF2 (o.scheme == KT_SCHEME_TRBDF2): stage 0 trapezoidal, r = Y + d h f_n in
-    //     YH (-> YF), stage 1 BDF2, r = w1 YF - w0 Y in YH (-> Y2); one FP32 factor of
+    //     YH (-> YF), stage 1 BDF2, r = w1 YF - w0 Y in YH; one FP32 factor of
     //     I - d h J serves both stages.  F0 holds f_n: f(Y) on the cell's first step,
     //     afterwards the previous step's stage relation (y_{n+1} - r)/(d h), which keeps
     //     the rounding of an evaluated rate (amplified by h k in the error estimate) out
@@ -637,81 +852,93 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
             const double dh = tr.d * h;
             bool ok = true;
             if (trs && !f0ok) {
-                const double T = ENERGY ? Y[ns] : T_iso;
-                ok = T > 0.0;
+                sync();
+                put(ys, Y);
+                sync();
+                const double Tc = ENERGY ? ys[ns] : T_iso;
+                ok = Tc > 0.0;
                 if (ok) {
-                    coefficients(T, Y);
-                    rows(Y, false);
-                    for (int i = lane; i < N; i += 32) F0[i] = W[i];
-                    __syncwarp();
+                    rates_rows(false);
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) F0[q] = W[q];
                     f0ok = true;
                 }
             }
             for (int stg = 0; ok && stg < nst; ++stg) {
-                const double *yb;
-                double *yt;
+                double YB[NQ];
                 double hph;
                 int fmode;
                 if (trs) {
-                    for (int i = lane; i < N; i += 32) {
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
                         if (stg == 0) {
-                            YH[i] = Y[i] + dh * F0[i];
-                            YF[i] = Y[i];
+                            YH[q] = fma(dh, F0[q], Y[q]);
+                            CUR[q] = Y[q];
                         } else {
-                            YH[i] = tr.w1 * YF[i] - tr.w0 * Y[i];
-                            Y2[i] = YF[i];
+                            YF[q] = CUR[q];
+                            YH[q] = fma(tr.w1, CUR[q], -__dmul_rn(tr.w0, Y[q]));
                         }
+                        YB[q] = YH[q];
                     }
-                    yb = YH;
-                    yt = stg == 0 ? YF : Y2;
                     hph = dh;
                     fmode = stg == 0 ? 2 : 0;
                 } else {
-                    const double *g = stg < 2 ? Y : (o.guess != KT_GUESS_PREV ? YF : YH);
-                    yt = stg == 0 ? YF : (stg == 1 ? YH : Y2);
-                    for (int i = lane; i < N; i += 32) yt[i] = g[i];
-                    yb = stg == 2 ? YH : Y;
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q) {
+                        if (stg == 0) {
+                            CUR[q] = Y[q];
+                        } else if (stg == 1) {
+                            YF[q] = CUR[q];
+                            CUR[q] = Y[q];
+                        } else {
+                            YH[q] = CUR[q];
+                            if (o.guess != KT_GUESS_PREV) CUR[q] = YF[q];
+                        }
+                        YB[q] = stg == 2 ? YH[q] : Y[q];
+                    }
                     hph = stg == 0 ? h : 0.5 * h;
                     fmode = 2 - stg;
                 }
-                __syncwarp();
-                ok = be_solve(yb, yt, hph, fmode);
+                sync();
+                put(ys, CUR);
+                ok = be_solve(YB, hph, fmode);
             }
             if (!ok) {
                 h *= 0.5;
                 if (h < o.h_min) return false;
                 continue;
             }
-            double s2 = 0.0;
-            if (trs) {
-                // local error estimate 2 C h (a0 f_n + a1 f_g + a2 f_{n+1}), the stage
-                // rates taken from the stage equations
-                const double inv = 1.0 / dh, ce = 2.0 * tr.C * h;
-                for (int i = lane; i < N; i += 32) {
-                    const double yn = Y[i], y1 = Y2[i], f0 = F0[i];
-                    const double fg = (YF[i] - yn) * inv - f0;
-                    const double f1 = (y1 - YH[i]) * inv;
-                    const double est = ce * (tr.a0 * f0 + tr.a1 * fg + tr.a2 * f1);
-                    const double sc = (i < ns ? atol_s : 0.0) + o.rtol * fmax(fabs(yn), fabs(y1));
-                    const double e = est / sc;
-                    s2 += e * e;
+            // local error: 2 C h (a0 f_n + a1 f_g + a2 f_{n+1}) with the stage rates taken from
+            // the stage equations, or the step-doubling difference; its weighted RMS
+            const double inv = trs ? 1.0 / dh : 0.0, ce = __dmul_rn(__dmul_rn(2.0, tr.C), h);
+            sync();
+#pragma unroll
+            for (int q = 0; q < NQ; ++q) {
+                const int i = own(q);
+                if (i >= N) continue;
+                const double yn = Y[q], y1 = CUR[q];
+                const double sc = fma(o.rtol, fmax(fabs(yn), fabs(y1)), i < ns ? atol_s : 0.0);
+                double est;
+                if (trs) {
+                    const double f0 = F0[q];
+                    const double fg = fma(__dadd_rn(YF[q], -yn), inv, -f0);
+                    const double f1 = __dmul_rn(__dadd_rn(y1, -YH[q]), inv);
+                    est = __dmul_rn(ce, fma(tr.a2, f1, fma(tr.a0, f0, __dmul_rn(tr.a1, fg))));
+                } else {
+                    est = __dadd_rn(y1, -YF[q]);
                 }
-            } else {
-                for (int i = lane; i < N; i += 32) {
-                    const double y = Y[i], y2 = Y2[i];
-                    const double sc = (i < ns ? atol_s : 0.0) + o.rtol * fmax(fabs(y), fabs(y2));
-                    const double e = (y2 - YF[i]) / sc;
-                    s2 += e * e;
-                }
+                fs[i] = est / sc;
             }
+            sync();
+            double s2 = 0.0;
+            for (int i = lane; i < N; i += 32) s2 = fma(fs[i], fs[i], s2);
             const double err = sqrt(wsum(s2) / N);
             if (err <= 1.0) {
-                const double inv = trs ? 1.0 / dh : 0.0;
-                for (int i = lane; i < N; i += 32) {
-                    if (trs) F0[i] = (Y2[i] - YH[i]) * inv;    // first same as last
-                    Y[i] = Y2[i];
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    if (trs) F0[q] = __dmul_rn(__dadd_rn(CUR[q], -YH[q]), inv);    // first same as last
+                    Y[q] = CUR[q];
                 }
-                __syncwarp();
                 ++nacc;
                 if (last) return true;
                 tt += h;
@@ -728,24 +955,29 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
         }
     };
 
-    // clip, then restore the element totals of the pre-processed input (Sec. 2.2.3)
+    // clip, then restore the element totals of the pre-processed input (Sec. 2.2.3); the
+    // state goes through fs, every warp forms the same sums
     auto post_process = [&]() -> bool {
         double b0[kMaxElements], r[kMaxElements], Mp[kMaxElements * kMaxElements];
-        for (int s = lane; s < ns; s += 32)
-            if (Y[s] < 0.0) Y[s] = 0.0;
-        __syncwarp();
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            if (own(q) < ns && Y[q] < 0.0) Y[q] = 0.0;
+        sync();
+        put(fs, Y);
+        sync();
         for (int e = 0; e < ne; ++e) {
             double pb = 0.0, pt = 0.0;
             for (int s = lane; s < ns; s += 32) {
                 const double v = yin(s);
-                pb += t.cnt[s * ne + e] * (v > 0.0 ? v : 0.0);
-                pt += t.cnt[s * ne + e] * Y[s];
+                pb = fma(t.cnt[s * ne + e], v > 0.0 ? v : 0.0, pb);
+                pt = fma(t.cnt[s * ne + e], fs[s], pt);
             }
             b0[e] = wsum(pb);
             r[e] = wsum(pt) - b0[e];
             for (int f = 0; f < ne; ++f) {
                 double pm = 0.0;
-                for (int s = lane; s < ns; s += 32) pm += t.cnt[s * ne + e] * t.cnt[s * ne + f] * Y[s];
+                for (int s = lane; s < ns; s += 32)
+                    pm = fma(__dmul_rn(t.cnt[s * ne + e], t.cnt[s * ne + f]), fs[s], pm);
                 Mp[e * ne + f] = wsum(pm);
             }
         }
@@ -782,22 +1014,32 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
             for (int j = i + 1; j < ne; ++j) s -= Mp[i * ne + j] * r[j];
             r[i] = s / Mp[i * ne + i];
         }
-        bool ok = true;
+        bool ok = !ENERGY || isfinite(fs[ns]);
         for (int s = lane; s < ns; s += 32) {
             double corr = 0.0;
-            for (int e = 0; e < ne; ++e) corr += t.cnt[s * ne + e] * r[e];
-            ok = ok && corr < 1.0;
-            Y[s] -= Y[s] * corr;
+            for (int e = 0; e < ne; ++e) corr = fma(t.cnt[s * ne + e], r[e], corr);
+            ok = ok && corr < 1.0 && isfinite(fma(-fs[s], corr, fs[s]));
         }
-        __syncwarp();
-        for (int i = lane; i < N; i += 32) ok = ok && isfinite(Y[i]);
-        return wall(ok);
+#pragma unroll
+        for (int q = 0; q < NQ; ++q)
+            if (own(q) < ns) {
+                double corr = 0.0;
+                for (int e = 0; e < ne; ++e) corr = fma(t.cnt[own(q) * ne + e], r[e], corr);
+                Y[q] = fma(-Y[q], corr, Y[q]);
+            }
+        return __all_sync(kFull, ok) != 0;
     };
 
     auto write_out = [&](int st, int nsub) {
-        for (int s = lane; s < ns; s += 32) a.y_out[static_cast<long long>(s) * nc + cell] = Y[s];
-        if (lane == 0) {
-            a.T_out[cell] = ENERGY ? Y[ns] : T_iso;
+        sync();   // every thread has read its inputs (in-place calls)
+#pragma unroll
+        for (int q = 0; q < NQ; ++q) {
+            const int i = own(q);
+            if (i < ns) a.y_out[static_cast<long long>(i) * nc + cell] = Y[q];
+            else if (ENERGY && i == ns) a.T_out[cell] = Y[q];
+        }
+        if (tid == 0) {
+            if (!ENERGY) a.T_out[cell] = T_iso;
             if (a.status) a.status[cell] = st;
             if (a.nsub) a.nsub[cell] = nsub;
             if (a.nnew) a.nnew[cell] = nnew;
@@ -808,9 +1050,11 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
         dtc = a.dt_cell ? a.dt_cell[cell] : a.dt;
         bool fin = isfinite(a.T_in[cell]) && dtc > 0.0 && isfinite(dtc);
         for (int s = lane; s < ns; s += 32) fin = fin && isfinite(yin(s));
-        if (!wall(fin)) {
-            for (int s = lane; s < ns; s += 32) a.y_out[static_cast<long long>(s) * nc + cell] = yin(s);
-            if (lane == 0) {
+        fin = __all_sync(kFull, fin) != 0;
+        if (!fin) {
+            sync();
+            for (int s = tid; s < ns; s += T) a.y_out[static_cast<long long>(s) * nc + cell] = yin(s);
+            if (tid == 0) {
                 a.T_out[cell] = a.T_in[cell];
                 if (a.status) a.status[cell] = KT_STATUS_NONFINITE;
                 if (a.nsub) a.nsub[cell] = 0;
@@ -819,20 +1063,23 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
             return;
         }
         load_pre();
+        sync();
+        put(fs, Y);
+        sync();
         double cvt = 0.0, b00 = 0.0;
         for (int s = lane; s < ns; s += 32) {
-            cvt += t.cv[s] * Y[s];
-            b00 += t.cnt[s * ne] * Y[s];
+            cvt = fma(t.cv[s], fs[s], cvt);
+            b00 = fma(t.cnt[s * ne], fs[s], b00);
         }
         cvt = wsum(cvt);
         b00 = wsum(b00);
         invCV = ENERGY ? 1.0 / cvt : 0.0;
         if (CVP) {
-#pragma unroll
             for (int k = 0; k < 10; ++k) {
                 double c = 0.0;
-                for (int s = lane; s < ns; s += 32) c += Y[s] * cvp[s * 10 + k];
-                cvc[k] = wsum(c);
+                for (int s = lane; s < ns; s += 32) c = fma(fs[s], cvp[s * 10 + k], c);
+                c = wsum(c);
+                if (tid == 0) cvc[k] = c;
             }
         }
         atol_s = (o.atol_mode == 1 && b00 > 0.0) ? o.atol * b00 : o.atol;
@@ -858,12 +1105,11 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
         if (!ENERGY) {
             const double lt = log_t(T_iso, nv.t_ref), invT = 1.0 / T_iso;
             const double lT = nv.ntab ? log(T_iso) : 0.0;
-            for (int r = lane; r < nr; r += 32) {
+            for (int r = tid; r < nr; r += T) {
                 double k, dk;
                 rate(r, T_iso, lt, lT, invT, k, dk);
                 K[r] = k;
             }
-            __syncwarp();
         }
         nnew = 0;
         int nacc = 0;
@@ -880,70 +1126,91 @@ __global__ void __launch_bounds__(kMaxWarps * 32, 2) warp_kernel(const LaunchArg
         } else {
             write_out(st, nacc);
         }
-        __syncwarp();
     };
 
-    if (PERSIST) {
+    if (a.persistent) {
         for (;;) {
             unsigned long long c = 0;
-            if (lane == 0) c = atomicAdd(&a.scratch->queue, 1ULL);
-            c = __shfl_sync(kFull, c, 0);
+            if constexpr (NW == 1) {
+                if (lane == 0) c = atomicAdd(&a.scratch->queue, 1ULL);
+                c = __shfl_sync(kFull, c, 0);
+            } else {
+                unsigned long long *next = reinterpret_cast<unsigned long long *>(wb + L.off_C);
+                sync();
+                if (tid == 0) *next = atomicAdd(&a.scratch->queue, 1ULL);
+                sync();
+                c = *next;
+                sync();
+            }
             if (c >= static_cast<unsigned long long>(nc)) break;
             cell = a.order ? static_cast<long long>(a.order[c]) : static_cast<long long>(c);
             process_cell();
         }
     } else {
-        cell = static_cast<long long>(blockIdx.x) * (blockDim.x >> 5) + wid;
+        cell = static_cast<long long>(blockIdx.x) * (blockDim.x / T) + team;
         if (cell < nc) process_cell();
     }
-    (void)h_fact;
 }
 
-template <bool ENERGY, bool F32, bool PERSIST>
+// Teams per block: one up to an SM's worth of cells, so that a small batch spreads over all
+// SMs, then as many as share the staged network within an SM's shared memory.
+template <int NW, int NQW, bool ENERGY, bool F32>
 int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
-    const WarpLayout L = warp_layout(a.nv.N, a.nv.nr, a.nv.energy, F32 ? 1 : 0, a.nv.bytes_warp,
-                                     F32 && a.o.scheme == KT_SCHEME_TRBDF2);
+    constexpr int NQ = NW == 1 ? NQW : 1, max_teams = (NW == 1 ? 8 : 16) / NW;
+    auto layout = [&](bool slim) {
+        return warp_layout(a.nv.N, a.nv.nr, a.nv.energy, F32 ? 1 : 0, a.nv.bytes_warp,
+                           !F32 || a.o.scheme == KT_SCHEME_TRBDF2, a.nv.nin_max, a.nv.cvpoly, slim);
+    };
+    WarpLayout L = layout(false);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     int smem_optin = 0, nsm = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    int warps = c.block_warps > 0 ? c.block_warps : 4;
-    if (warps > kMaxWarps) warps = kMaxWarps;
-    while (warps > 1 && L.base + warps * L.warp_bytes > smem_optin) --warps;
-    const size_t smem = static_cast<size_t>(L.base) + static_cast<size_t>(warps) * L.warp_bytes;
+    if (L.base + L.warp_bytes > smem_optin) L = layout(true);
+    const long long per_sm = (a.ncells + nsm - 1) / nsm;
+    int teams = c.block_warps > 0 ? c.block_warps / NW : (NW == 1 ? 4 : max_teams);
+    if (c.block_warps <= 0 && teams > per_sm) teams = static_cast<int>(per_sm);
+    if (teams > max_teams) teams = max_teams;
+    if (teams < 1) teams = 1;
+    while (teams > 1 && L.base + teams * L.warp_bytes > smem_optin) --teams;
+    const size_t smem = static_cast<size_t>(L.base) + static_cast<size_t>(teams) * L.warp_bytes;
     if (smem > static_cast<size_t>(smem_optin)) return cudaErrorInvalidConfiguration;
-    auto kern = warp_kernel<ENERGY, F32, PERSIST>;
+    auto kern = warp_kernel<NW, NQ, NQW, ENERGY, F32>;
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
     if (e != cudaSuccess) return e;
-    const int threads = warps * 32;
-    long long blocks;
-    if (PERSIST) {
-        int per_sm = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, threads, smem);
+    const int threads = teams * NW * 32;
+    long long blocks = (a.ncells + teams - 1) / teams;
+    if (a.persistent) {
+        int fit = 0;
+        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&fit, kern, threads, smem);
         if (e != cudaSuccess) return e;
-        if (per_sm < 1) per_sm = 1;
-        if (c.blocks_per_sm > 0 && c.blocks_per_sm < per_sm) per_sm = c.blocks_per_sm;
-        blocks = static_cast<long long>(per_sm) * nsm;
-        const long long need = (a.ncells + warps - 1) / warps;
-        if (blocks > need) blocks = need;
-    } else {
-        blocks = (a.ncells + warps - 1) / warps;
+        if (fit < 1) fit = 1;
+        if (c.blocks_per_sm > 0 && c.blocks_per_sm < fit) fit = c.blocks_per_sm;
+        if (blocks > static_cast<long long>(fit) * nsm) blocks = static_cast<long long>(fit) * nsm;
     }
     if (blocks < 1) return cudaSuccess;
     kern<<<static_cast<unsigned>(blocks), threads, smem, s>>>(a, L);
     return cudaGetLastError();
 }
 
-// Dispatch over the compile-time options for one form of the iteration matrix.
+// Dispatch over the compile-time options for one form of the iteration matrix.  Up to 32
+// unknowns one warp holds a row per lane and four would mostly wait for each other
+// (32 species, dt 1e8 s, one | four warps: 300 cells 163 | 159 ms, 2,049 cells 134 | 189,
+// 8,192 cells 207 | 475); beyond, the team is faster at every size (65 unknowns, dt 1e-9 s:
+// 1,024 cells 546 | 291 ms; 8,192 cells at 1e-10 s 615 | 405).
+template <bool F32, bool ENERGY>
+int launch_warp_size(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
+{
+    return a.nv.N <= 32 ? launch_t<1, 1, ENERGY, F32>(a, c, s) : launch_t<4, 3, ENERGY, F32>(a, c, s);
+}
+
 template <bool F32>
 int launch_warp_form(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
-    const bool en = a.nv.energy != 0, per = c.persistent != 0;
-    if (en) return per ? launch_t<true, F32, true>(a, c, s) : launch_t<true, F32, false>(a, c, s);
-    return per ? launch_t<false, F32, true>(a, c, s) : launch_t<false, F32, false>(a, c, s);
+    return a.nv.energy ? launch_warp_size<F32, true>(a, c, s) : launch_warp_size<F32, false>(a, c, s);
 }
 
 }  // namespace
