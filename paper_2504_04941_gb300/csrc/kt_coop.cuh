@@ -538,7 +538,7 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
                 if (u0 & kCoopEnd) {
                     const unsigned to = *next;
                     next += G;
-                    if (need) M[to] = (u0 & kCoopDiag) ? v + R(1) : v;
+                    if (need) M[to] = v;
                     v = R(0);
                 }
                 u0 = u1;
@@ -567,7 +567,8 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
                     big = m > big ? m : big;
                 }
                 ok = ok && big > R(0);
-                if (need) V[i] = big > R(0) ? R(1) / big : R(1);
+                const R inv = R(1) / (need && big > R(0) ? big : R(1));
+                if (need) V[i] = inv;
             }
             unsigned long long pm = 0xfedcba9876543210ULL;
             __syncwarp();
@@ -617,7 +618,7 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
                 const unsigned long long df = ((pm >> (4 * j)) ^ (pm >> (4 * imax))) & 15ULL;
                 pm ^= (df << (4 * j)) ^ (df << (4 * imax));
                 __syncwarp();
-                const R rinv = R(1) / M[j * LD + j];
+                const R rinv = R(1) / (need ? M[j * LD + j] : R(1));
                 __syncwarp();
                 for (int i = j + 1 + gl; i < N; i += G)
                     if (need) M[i * LD + j] *= rinv;
@@ -759,9 +760,10 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
             const double tol = fma(o.newton_rtol, fabs(y), own[q] < ns ? natol : 0.0);
             if (!abs_le(d[q], tol)) convl = false;
             if constexpr (F32) {
-                const float ad = fabsf(df[q]), tf = static_cast<float>(tol);
+                // (idle groups divide by 1, see above)
+                const float ad = run ? fabsf(df[q]) : 0.0f, tf = run ? static_cast<float>(tol) : 1.0f;
                 const float e = __fdiv_rn(ad, fmaxf(tf, 1e-37f));
-                const float trl = __fmul_rn(rtol_f, fabsf(y32));
+                const float trl = run ? __fmul_rn(rtol_f, fabsf(y32)) : 1.0f;
                 const float er = __fdiv_rn(ad, fmaxf(trl, 1e-37f));
                 dmax = e > dmax ? e : dmax;
                 dmaxr = er > dmaxr ? er : dmaxr;
@@ -781,7 +783,7 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
                     dmaxr = fmaxf(dmaxr, __shfl_xor_sync(kFull, dmaxr, s));
                 }
             }
-            if (!conv && !bad && luok && it > 0) {
+            if (!conv && !bad && luok && it > 0 && run) {
                 const float th = dmaxr / dprevr;
                 if (th < 0.5f && th / (1.0f - th) * dmaxr <= 1.0f) conv = true;
             }

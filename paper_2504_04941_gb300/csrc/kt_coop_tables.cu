@@ -82,13 +82,14 @@ bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *n
             if (energy) ent[ns * N + col].push_back(d | (partial(nin_max + 1, r) << 16));
         }
     const unsigned pad_row = 8u * nr;   // rate 0 with coefficient 0; partial 0 with coefficient 0
-    auto close = [](Terms &list, unsigned pad, unsigned flags) {
+    auto close = [](Terms &list, unsigned pad) {
         if (list.empty()) list.push_back(pad);
-        list.back() |= kCoopEnd | flags;
+        list.back() |= kCoopEnd;
     };
     for (int i = 0; i < N; ++i) {
-        close(rows[i], pad_row, 0u);
-        for (int j = 0; j < N; ++j) close(ent[i * N + j], 0u, i == j ? kCoopDiag : 0u);
+        close(rows[i], pad_row);
+        ent[i * N + i].push_back(rb | (rb << 16));   // the identity: + 1 * 1 after the updates
+        for (int j = 0; j < N; ++j) close(ent[i * N + j], 0u);
     }
     const std::vector<int> row_lane = deal(rows, G, NC), ent_lane = deal(ent, G, N * N);
     std::vector<unsigned> rp, jp;

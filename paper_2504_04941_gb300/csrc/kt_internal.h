@@ -85,7 +85,6 @@ enum DevError : int { kDevErrNone = 0, kDevErrTma = 1 };
 // and of its coefficient (16..29: +1, -1 or the heat over C_V) in the cell's partials.
 constexpr unsigned kCoopOffset = 0x3fffu;
 constexpr unsigned kCoopEnd = 1u << 15;     // last term of a row or entry
-constexpr unsigned kCoopDiag = 1u << 14;    // ... whose entry is on the diagonal
 constexpr int kCoopConst = 4;               // 0, 1, -1 before the partials
 constexpr int kCoopMaxReactions = 400;    // offsets stay within 14 bits (5 kinds x 8 bytes)
 constexpr int kCoopPad = 2;                 // padding steps after each program (prefetch)

@@ -114,8 +114,7 @@ def test_programs_replay_the_reaction_loop(probe, N, energy, nr, G, fp32):
             v = ft(v + part[((u >> 16) & 0x3fff) // rb] * part[(u & 0x3fff) // rb])
             if u & 0x8000:
                 at = int(to[k * G + l])
-                gotM[at // LD, at % LD] = ft(v + ft(1)) if u & 0x4000 else v
-                assert bool(u & 0x4000) == (at // LD == at % LD)
+                gotM[at // LD, at % LD] = v
                 v, k, seen = ft(0), k + 1, seen + 1
     assert seen == N * N
     assert np.array_equal(gotf, f) and np.array_equal(gotM, M)
