@@ -75,6 +75,8 @@ struct kt_network {
     // they follow the tables (view.bytes_total) in the blob; -1 where the network has none
     std::array<int, 8> coop_off{{-1, -1, -1, -1, -1, -1, -1, -1}};
     std::array<kt::CoopTab, 8> coop_tab{};
+    // Jacobian program of the larger-network kernels (FP64 form, FP32-LU), also in the blob
+    std::array<int, 2> jac_off{{-1, -1}}, jac_steps{{0, 0}}, jac_bytes{{0, 0}};
     const kt_mlp *mlp = nullptr;                  // attached learned-guess MLP (not owned)
     std::mutex mu;
     std::map<int, unsigned char *> dev_blob;      // device ordinal -> device copy
@@ -424,6 +426,30 @@ void build_blob(kt_network *n)
     }
 }
 
+// Appends the Jacobian programs of the larger-network kernels to the blob.
+void build_team(kt_network *n)
+{
+    const int N = n->view.N, T = N <= 32 ? 32 : 128;
+    if (N > kt::kWarpMaxN || n->nr < 1) return;
+    std::vector<int> rp(n->ns + 1), re(n->view.nent);
+    std::memcpy(rp.data(), n->blob.data() + n->view.off_rp, 4 * rp.size());
+    if (!re.empty()) std::memcpy(re.data(), n->blob.data() + n->view.off_re, 4 * re.size());
+    std::vector<unsigned> prog;
+    for (int f = 0; f < 2; ++f) {
+        const int LD = kt::warp_layout(N, n->nr, n->energy, f, 0).LD;
+        const int steps = kt::team_jacobian(n->ns, n->nr, n->energy, n->nin.data(),
+                                            reinterpret_cast<const int(*)[kt::kMaxSide]>(n->in.data()), rp, re, LD, T,
+                                            &prog);
+        if (!steps) continue;
+        n->jac_off[f] = static_cast<int>(n->blob.size());
+        n->jac_steps[f] = steps;
+        n->jac_bytes[f] = static_cast<int>(4 * prog.size());
+        const unsigned char *b = reinterpret_cast<const unsigned char *>(prog.data());
+        n->blob.insert(n->blob.end(), b, b + n->jac_bytes[f]);
+        n->blob.resize((n->blob.size() + 15) & ~static_cast<size_t>(15));
+    }
+}
+
 // Appends the per-lane programs of every group size to the blob.
 void build_coop(kt_network *n)
 {
@@ -524,6 +550,7 @@ int kt_network_load(const char *path, kt_network **out)
     }
     build_blob(n);
     build_coop(n);
+    build_team(n);
     *out = n;
     return KT_OK;
 }
@@ -649,6 +676,11 @@ int integrate_impl(const kt_network *net, int64_t ncells, const double *y_in, co
         a.coop_g = grp;
         if (!kt::coop_fits(a, c)) a.coop = nullptr;
     }
+    const int f32 = opts->form == KT_FORM_FP32LU;
+    if (cpw == 1 && net->jac_off[f32] >= 0) {
+        a.jac = reinterpret_cast<const unsigned *>(blob + net->jac_off[f32]);
+        a.jac_steps = net->jac_steps[f32];
+    }
     int ce = a.coop ? kt::launch_coop(a, c, cuda_stream)
                     : cpw == 32 ? kt::launch_lane(a, c, cuda_stream) : kt::launch_warp(a, c, cuda_stream);
     if (ce != 0) return cuda_fail(static_cast<cudaError_t>(ce), "integrate kernel launch");
@@ -700,7 +732,8 @@ int kt::network_element_basis(const kt_network *net, double *Vr, int *ns_out, in
 int kt::prepare_launch(const kt_network *net, int64_t ncells, const double *y_in, const double *T_in,
                        const double *rho, double dt, const kt_options *opts, double *y_out, double *T_out,
                        int32_t *status, int32_t *n_substeps, int32_t *n_newton, kt::LaunchArgs *a,
-                       kt::LaunchCfg *c, const unsigned char **host_blob)
+                       kt::LaunchCfg *c, const unsigned char **host_blob, const unsigned char **host_jac,
+                       int *jac_bytes)
 {
     if (!net) return fail(KT_EINVAL, "NULL network");
     if (ncells < 0 || !(dt > 0) || !std::isfinite(dt)) return fail(KT_EINVAL, "bad ncells or dt");
@@ -730,6 +763,14 @@ int kt::prepare_launch(const kt_network *net, int64_t ncells, const double *y_in
     a->persistent = opts->persistent != 0;
     *c = kt::LaunchCfg{opts->form, opts->persistent, opts->block_warps, opts->blocks_per_sm, cpw, opts->lane_variant};
     *host_blob = net->blob.data();
+    const int f32 = opts->form == KT_FORM_FP32LU;
+    *host_jac = nullptr;
+    *jac_bytes = 0;
+    if (cpw == 1 && net->jac_off[f32] >= 0) {
+        *host_jac = net->blob.data() + net->jac_off[f32];
+        *jac_bytes = net->jac_bytes[f32];
+        a->jac_steps = net->jac_steps[f32];
+    }
     return KT_OK;
 }
 

@@ -1,4 +1,5 @@
-// kt_coop_tables.cu -- per-lane programs of the kernels with G lanes per cell (host code).
+// kt_coop_tables.cu -- per-lane programs of the kernels with G lanes per cell, and the
+// Jacobian program of the larger-network kernels (host code).
 //
 // A program is a list of terms per lane; the G lists run side by side, padded to the
 // longest.  Rows of f (and entries of the iteration matrix) are dealt to the lanes
@@ -121,6 +122,36 @@ bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *n
     for (int r = 0; r < nr; ++r) cf.push_back(-dH[r]);
     std::memcpy(bytes->data() + tab->off_coef, cf.data(), 8 * cf.size());
     return true;
+}
+
+int team_jacobian(int ns, int nr, int energy, const int *nin, const int (*in)[kMaxSide], const std::vector<int> &rp,
+                  const std::vector<int> &re, int LD, int T, std::vector<unsigned> *prog)
+{
+    const int N = ns + energy;
+    int nin_max = 1;
+    for (int r = 0; r < nr; ++r) nin_max = std::max(nin_max, nin[r]);
+    const int zero = nr * (nin_max + energy);   // the partial that is always 0
+    if (zero > static_cast<int>(kTermIndex) || N * LD > static_cast<int>(kTermIndex)) return 0;
+    std::vector<Terms> ent(static_cast<size_t>(ns) * N);
+    for (int s = 0; s < ns; ++s)
+        for (int e = rp[s]; e < rp[s + 1]; ++e) {
+            const int r = re[e] >> 8;
+            const unsigned sign = (re[e] & 0x80) ? kTermMinus : 0u;
+            for (int c = 0; c < nin[r]; ++c)
+                ent[s * N + in[r][c]].push_back(sign | static_cast<unsigned>(c * nr + r));
+            if (energy) ent[s * N + ns].push_back(sign | static_cast<unsigned>(nin_max * nr + r));
+        }
+    for (int s = 0; s < ns; ++s)
+        for (int m = 0; m < N; ++m) {
+            Terms &list = ent[s * N + m];
+            if (list.empty()) list.push_back(static_cast<unsigned>(zero));
+            list.back() |= kTermEnd | (static_cast<unsigned>(m * LD + s) << kTermPlace);
+        }
+    const int steps = pack(ent, deal(ent, T, ns * N), T, static_cast<unsigned>(zero), prog);
+    const int padded = (steps + 7) & ~7;
+    prog->resize(static_cast<size_t>(padded + 8) * T, static_cast<unsigned>(zero));
+    std::fill(prog->begin() + static_cast<size_t>(steps) * T, prog->end(), static_cast<unsigned>(zero));
+    return padded;
 }
 
 }  // namespace kt

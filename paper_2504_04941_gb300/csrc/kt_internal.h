@@ -94,6 +94,12 @@ constexpr int coop_nm(int N) { return N == 3 ? 3 : (N == 11 ? 11 : kLaneMaxN); }
 constexpr int coop_ld(int NM) { return (NM + 3) & ~3; }
 constexpr int kCoopMaxWarps = 4;
 
+// Jacobian program of the larger-network kernels: [step][thread] terms, a term being the
+// partial's index (bits 0..13), the entry's place in the matrix (14..27, with kTermEnd) and
+// the sign; padded to a multiple of eight steps and eight more for the prefetch.
+constexpr unsigned kTermIndex = 0x3fffu, kTermEnd = 1u << 28, kTermMinus = 1u << 31;
+constexpr int kTermPlace = 14;
+
 struct CoopTab {
     int n_row, n_jac;      // steps of the row and matrix programs
     int off_row, off_jac;  // byte offsets of the uint32 [step][G] programs (the owned
@@ -110,6 +116,8 @@ struct LaunchArgs {
     const unsigned char *coop;   // device programs of the chosen group size (null: one cell per lane)
     CoopTab coop_tab;
     int coop_g;                  // lanes per cell of those programs
+    const unsigned *jac;         // larger networks: Jacobian program (null: rows walk their lists)
+    int jac_steps;
     int persistent;
     DevOpts o;
     double dt;
@@ -286,7 +294,7 @@ inline WarpLayout warp_layout(int N, int nr, int energy, int fp32, int blob_byte
     L.off_W = take(N * 8);
     L.off_RW = take(nr * 8);
     L.off_K = energy && !slim ? 0 : take(nr * 8);
-    L.off_D = slim ? -1 : take(nr * r * (nin_max + (energy ? 1 : 0)));
+    L.off_D = slim ? -1 : take((nr * (nin_max + (energy ? 1 : 0)) + 1) * r);
     L.off_CV = cvpoly ? take(10 * 8) : 0;
     L.off_C = N > 32 ? take(2 * 3 * 4 * 4) : 0;
     L.warp_bytes = (o + 127) & ~127;
@@ -311,7 +319,7 @@ const unsigned char *mlp_device_block(const kt_mlp *m, int *nin, int *nout, int 
 int prepare_launch(const kt_network *net, int64_t ncells, const double *y_in, const double *T_in,
                    const double *rho, double dt, const kt_options *opts, double *y_out, double *T_out,
                    int32_t *status, int32_t *n_substeps, int32_t *n_newton, LaunchArgs *a, LaunchCfg *c,
-                   const unsigned char **host_blob);
+                   const unsigned char **host_blob, const unsigned char **host_jac, int *jac_bytes);
 
 // Orthonormal basis Vr [ns][rank] of the element matrix's row space (rank <= 8).
 int network_element_basis(const kt_network *net, double *Vr, int *ns, int *rank);
@@ -327,6 +335,11 @@ int launch_schedule(const int *count, long long ncells, unsigned *work, int *ord
 bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *nout, const int (*in)[kMaxSide],
                  const int (*out)[kMaxSide], const double *dH, int fp32, int G, CoopTab *tab,
                  std::vector<unsigned char> *bytes);
+// Jacobian program of the larger-network kernels (kt_coop_tables.cu): T threads per cell,
+// column stride LD; rp / re: the species' lists of (reaction << 8 | +-1).  Returns the steps
+// (without the prefetch padding), 0 if an index does not fit.
+int team_jacobian(int ns, int nr, int energy, const int *nin, const int (*in)[kMaxSide], const std::vector<int> &rp,
+                  const std::vector<int> &re, int LD, int T, std::vector<unsigned> *prog);
 // Lanes per cell for this call (0: one cell per lane).
 int coop_group(const LaunchArgs &a, const LaunchCfg &c);
 // Whether a warp's cells fit in a block's shared memory beside the programs.

@@ -71,9 +71,10 @@ extern "C" KT_API int kt_integrate_noalloc(const kt_network *net, int64_t ncells
     }
     kt::LaunchArgs a{};
     kt::LaunchCfg c{};
-    const unsigned char *host_tables = nullptr;
+    const unsigned char *host_tables = nullptr, *host_jac = nullptr;
+    int jac_bytes = 0;
     int rc = kt::prepare_launch(net, ncells, y_in, T_in, rho, dt, opts, y_out, T_out, status, n_substeps,
-                                n_newton, &a, &c, &host_tables);
+                                n_newton, &a, &c, &host_tables, &host_jac, &jac_bytes);
     if (rc) return rc;
     const size_t need = kTablesOffset + static_cast<size_t>(a.nv.bytes_total);
     if (need > kNoAllocBytes) {
@@ -96,6 +97,11 @@ extern "C" KT_API int kt_integrate_noalloc(const kt_network *net, int64_t ncells
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(area + kTablesOffset, host_tables, static_cast<size_t>(a.nv.bytes_total),
                             cudaMemcpyHostToDevice, s);
+    // the Jacobian program follows the tables where it fits; without it the rows walk their lists
+    if (e == cudaSuccess && host_jac && need + static_cast<size_t>(jac_bytes) <= kNoAllocBytes) {
+        e = cudaMemcpyAsync(area + need, host_jac, static_cast<size_t>(jac_bytes), cudaMemcpyHostToDevice, s);
+        a.jac = reinterpret_cast<const unsigned *>(area + need);
+    }
     if (e == cudaSuccess) e = cudaMemsetAsync(status, 0xff, static_cast<size_t>(ncells) * sizeof(int32_t), s);
     if (e != cudaSuccess) {
         char msg[256];

@@ -8,9 +8,10 @@
 //   rates          threads over reactions (modified Arrhenius, Sec. 2.2.1): the rate w_r and,
 //                  when a Jacobian is wanted, its partial derivatives, each formed once in
 //                  FP64 and rounded once (the rows below only add them);
-//   f and J rows   threads over species rows, each walking its own list of (reaction, +-1)
-//                  entries, so every row is accumulated by one thread in a fixed order:
-//                  deterministic, no atomics (Eq. method-jacobian);
+//   f and J rows   threads over species rows of f, each walking its own list of (reaction,
+//                  +-1) entries; threads over the entries of J, each entry's terms summed by
+//                  one thread in the same order (a program the host lays out once): fixed
+//                  orders, no atomics (Eq. method-jacobian);
 //   T row          threads over columns: J_T,m = -sum_s h_s J_s,m / C_V, and I - h J of the
 //                  column in the same pass;
 //   LU             right-looking with the implicit-scaled row pivoting of Algorithm
@@ -72,14 +73,12 @@ __device__ __forceinline__ double log_t(double T, double t_ref)
 __device__ __forceinline__ void arrhenius(const NetS &t, int r, double lt, double invT, double &k, double &dk)
 {
     const double b = t.b[r], th = t.th[r];
-    const double arg = b * lt - th * invT;
-    if (below_m700(arg)) {
-        k = 0.0;
-        dk = 0.0;
-    } else {
-        k = t.A[r] * tang_exp(arg, t.ex);
-        dk = k * (b + th * invT) * invT;
-    }
+    // (no branch: the exponentials of two reactions run interleaved)
+    const double arg = fma(b, lt, -__dmul_rn(th, invT));
+    const bool zero = below_m700(arg);
+    const double v = __dmul_rn(t.A[r], tang_exp(zero ? -700.0 : arg, t.ex));
+    k = zero ? 0.0 : v;
+    dk = __dmul_rn(__dmul_rn(k, fma(th, invT, b)), invT);
 }
 
 // phi(tau) = (1 - e^-tau)/tau of Eq. photo-reaction-single and its derivative; below
@@ -198,9 +197,11 @@ __device__ __forceinline__ int pivot_row(const double (&c)[NQW], int lane)
 }
 
 // NW warps per cell, NQ components per thread (thread t owns t, t + 32 NW, ...), NQW rows
-// per lane of one warp (N <= 32 NQW).
+// per lane of one warp (N <= 32 NQW).  Twelve single-warp teams per SM with 168 registers
+// rather than sixteen with 128 (32 species, dt 1e8 s: 1,000 cells 111 | 116 ms, 2,049 cells
+// 120 | 122, 4,096 cells 135 | 139, 8,192 cells 203 | 196).
 template <int NW, int NQ, int NQW, bool ENERGY, bool F32>
-__global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_kernel(const LaunchArgs a, const WarpLayout L)
+__global__ void __launch_bounds__(NW == 1 ? 128 : 512, NW == 1 ? 3 : 1) warp_kernel(const LaunchArgs a, const WarpLayout L)
 {
     using R = typename std::conditional<F32, float, double>::type;
     constexpr int T = 32 * NW, VW = 16 / sizeof(R);
@@ -266,6 +267,7 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
     double tab_w = 0.0, ph_F = 1.0, ph_dl = 0.0, ph_phi = 1.0, ph_dphi = 0.0;
     const int nin_max = nv.nin_max, kT = nin_max;   // kinds of partials: reactants, then T
     const bool slim = L.off_D < 0;                  // no room for partials: K and dk/dT (in ws) instead
+    if (!slim && tid == 0) D[nr * (nin_max + (ENERGY ? 1 : 0))] = R(0);   // the partial of padding terms
 
     // k and dk/dT of reaction r at T (lt = ln(T/T_ref), lT = ln T); photo-reactions take
     // the current phi(tau) (dk/dT = 0)
@@ -333,7 +335,7 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
             invT = 1.0 / Tc;
             lT = nv.ntab ? log(Tc) : 0.0;
         }
-        for (int r = tid; r < nr; r += T) {
+        auto reaction = [&](int r, bool on) {   // rate (and partials) of reaction r, kept if on
             double k, dk = 0.0;
             if (ENERGY) rate(r, Tc, lt, lT, invT, k, dk);
             else k = nv.nphoto && rtype[r] == 2 ? ph_F * sigr[r] * ph_phi : K[r];
@@ -347,6 +349,7 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
                 y2 = nin > 2 ? ys[(ix >> 32) & 0xff] : 1.0;
                 w = __dmul_rn(w, y2);
             }
+            if (!on) return;
             ws[r] = w;
             if (wantJ && slim) {
                 if (ENERGY) {
@@ -370,6 +373,17 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
                     D[kT * nr + r] = static_cast<R>(dT);
                 }
             }
+        };
+        if (ENERGY && !nv.special) {
+            // two reactions at a time: the second's loads and integer work hide behind the
+            // first's FP64 instructions
+            for (int r = tid; r < nr; r += 2 * T) {
+                const bool two = r + T < nr;
+                reaction(r, true);
+                reaction(two ? r + T : r, two);
+            }
+        } else {
+            for (int r = tid; r < nr; r += T) reaction(r, true);
         }
         sync();
         // f: every species row adds +-w_r per list entry (every entry has a coefficient of
@@ -395,80 +409,83 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
             }
             W[q] = f;
         }
-        if (wantJ) {
+        if (wantJ && !slim) {
+            // every entry of the species rows is the sum of its terms +-D in list order, formed by
+            // one thread (kt_coop_tables.cu); the program streams from L2, eight steps ahead.  (Rows
+            // walking their lists, read-modify-write: 65 unknowns 13.0k cycles per iteration,
+            // this 6.8k; 32 unknowns 3.8k | 2.5k.)
+            const unsigned *prog = a.jac + tid;
+            R v = R(0);
+            unsigned u[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) u[e] = __ldg(prog + e * T);
+            for (int e0 = 0; e0 < a.jac_steps; e0 += 8) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const unsigned c = u[e];
+                    u[e] = __ldg(prog + (e0 + 8 + e) * T);
+                    const R d = D[c & kTermIndex];
+                    if constexpr (F32) v += __uint_as_float(__float_as_uint(d) ^ (c & kTermMinus));
+                    else v += __hiloint2double(__double2hiint(d) ^ static_cast<int>(c & kTermMinus), __double2loint(d));
+                    if (c & kTermEnd) {
+                        J[(c >> kTermPlace) & kTermIndex] = v;
+                        v = R(0);
+                    }
+                }
+            }
+            if (nv.nphoto) {
+                // dw/dn_m of a photo rate through tau: + (sum) sigma_m for every absorber m, the
+                // sum over the row's photo reactions of nu F sigma_r n_i phi' dl
+                sync();
+                for (int s = tid; s < ns; s += T) {
+                    double gph = 0.0;
+                    const int e1 = t.rp[s + 1];
+                    for (int e = t.rp[s]; e < e1; ++e) {
+                        const int ent = t.re[e], r = ent >> 8;
+                        if (rtype[r] == 2) {
+                            const int i0 = static_cast<int>((t.idx[r] >> 16) & 0xff);
+                            const double g = ph_F * sigr[r] * ys[i0] * ph_dphi * ph_dl;
+                            gph += (ent & 0x80) ? -g : g;
+                        }
+                    }
+                    if (gph != 0.0)
+                        for (int m = 0; m < ns; ++m) {
+                            if constexpr (F32) J[m * LD + s] += static_cast<float>(__dmul_rn(gph, sigs[m]));
+                            else J[m * LD + s] = fma(gph, sigs[m], J[m * LD + s]);
+                        }
+                }
+            }
+        } else if (wantJ) {
             for (int s = tid; s < ns; s += T) {
                 R *row = J + s;   // entry m of the row at m * LD
                 for (int m = 0; m < N; ++m) row[m * LD] = R(0);
-                const int e0 = t.rp[s], e1 = t.rp[s + 1];
-                double gph = 0.0;    // photo: sum over the row's photo reactions of nu F sigma_r n_i phi' dl
+                const int e1 = t.rp[s + 1];
+                double gph = 0.0, f = 0.0;
                 R aT = R(0);
-                // an entry's reaction and partials are loaded while the one before it updates
-                // the row (what remains is the row's own read-modify-write chain)
-                struct Entry {
-                    int ent;
-                    unsigned long long ix;
-                    R d0, d1, dT;
-                };
-                double f = 0.0;
-                auto load = [&](int e) {
-                    Entry n{};
-                    if (e < e1) {
-                        n.ent = t.re[e];
-                        const int r = n.ent >> 8;
-                        n.ix = t.idx[r];
-                        if (slim) return n;
-                        n.d0 = D[r];
-                        if (nin_max > 1) n.d1 = D[nr + r];
-                        if (ENERGY) n.dT = D[kT * nr + r];
-                    }
-                    return n;
-                };
-                Entry n = load(e0);
-                for (int e = e0; e < e1; ++e) {
-                    Entry c = n;
-                    R d2 = R(0);
-                    n = load(e + 1);
-                    const int nin = static_cast<int>(c.ix & 0x7f);
-                    const int i0 = static_cast<int>((c.ix >> 16) & 0xff), i1 = static_cast<int>((c.ix >> 24) & 0xff);
-                    if (slim) {
-                        const int r = c.ent >> 8;
-                        const double k = K[r], y0 = ys[i0], y1 = nin > 1 ? ys[i1] : 1.0;
-                        const double y2 = nin > 2 ? ys[(c.ix >> 32) & 0xff] : 1.0, p01 = __dmul_rn(y0, y1);
-                        const double w = __dmul_rn(__dmul_rn(k, p01), y2);
-                        f += (c.ent & 0x80) ? -w : w;
-                        c.d0 = static_cast<R>(__dmul_rn(__dmul_rn(k, y1), y2));
-                        c.d1 = static_cast<R>(__dmul_rn(__dmul_rn(k, y0), y2));
-                        d2 = static_cast<R>(__dmul_rn(k, p01));
-                        if (ENERGY) c.dT = static_cast<R>(__dmul_rn(__dmul_rn(ws[r], p01), y2));
-                    } else if (nin > 2) {
-                        d2 = D[2 * nr + (c.ent >> 8)];
-                    }
-                    const R sg = (c.ent & 0x80) ? R(-1) : R(1);   // fma(+-1, d, a) = a +- d
-                    if (nin == 2 && i0 != i1) {
-                        // the two entries differ: both loaded, then both stored
-                        const R a0 = row[i0 * LD], a1 = row[i1 * LD];
-                        row[i0 * LD] = fma_t(sg, c.d0, a0);
-                        row[i1 * LD] = fma_t(sg, c.d1, a1);
-                    } else {
-                        const int i2 = static_cast<int>((c.ix >> 32) & 0xff);
-                        row[i0 * LD] = fma_t(sg, c.d0, row[i0 * LD]);
-                        if (nin > 1) row[i1 * LD] = fma_t(sg, c.d1, row[i1 * LD]);
-                        if (nin > 2) row[i2 * LD] = fma_t(sg, d2, row[i2 * LD]);
-                    }
-                    if (ENERGY) aT = fma_t(sg, c.dT, aT);
-                    if (nv.nphoto && rtype[c.ent >> 8] == 2) {
-                        const double g = ph_F * sigr[c.ent >> 8] * ys[i0] * ph_dphi * ph_dl;
-                        gph += (c.ent & 0x80) ? -g : g;
+                for (int e = t.rp[s]; e < e1; ++e) {
+                    const int ent = t.re[e], r = ent >> 8;
+                    const unsigned long long ix = t.idx[r];
+                    const int nin = static_cast<int>(ix & 0x7f);
+                    const int i0 = static_cast<int>((ix >> 16) & 0xff), i1 = static_cast<int>((ix >> 24) & 0xff),
+                              i2 = static_cast<int>((ix >> 32) & 0xff);
+                    const R sg = (ent & 0x80) ? R(-1) : R(1);   // fma(+-1, d, a) = a +- d
+                    const double k = K[r], y0 = ys[i0], y1 = nin > 1 ? ys[i1] : 1.0, y2 = nin > 2 ? ys[i2] : 1.0;
+                    const double p01 = __dmul_rn(y0, y1), w = __dmul_rn(__dmul_rn(k, p01), y2);
+                    f += (ent & 0x80) ? -w : w;
+                    row[i0 * LD] = fma_t(sg, static_cast<R>(__dmul_rn(__dmul_rn(k, y1), y2)), row[i0 * LD]);
+                    if (nin > 1) row[i1 * LD] = fma_t(sg, static_cast<R>(__dmul_rn(__dmul_rn(k, y0), y2)), row[i1 * LD]);
+                    if (nin > 2) row[i2 * LD] = fma_t(sg, static_cast<R>(__dmul_rn(k, p01)), row[i2 * LD]);
+                    if (ENERGY) aT = fma_t(sg, static_cast<R>(__dmul_rn(__dmul_rn(ws[r], p01), y2)), aT);
+                    if (nv.nphoto && rtype[r] == 2) {
+                        const double g = ph_F * sigr[r] * y0 * ph_dphi * ph_dl;
+                        gph += (ent & 0x80) ? -g : g;
                     }
                 }
                 if (ENERGY) row[ns * LD] = aT;
-                if (slim) {
-                    fs[s] = f;
+                fs[s] = f;
 #pragma unroll
-                    for (int q = 0; q < NQ; ++q)
-                        if (own(q) == s) W[q] = f;
-                }
-                // dw/dn_m of a photo rate through tau: + (sum) sigma_m for every absorber m
+                for (int q = 0; q < NQ; ++q)
+                    if (own(q) == s) W[q] = f;
                 if (gph != 0.0)
                     for (int m = 0; m < ns; ++m) {
                         if constexpr (F32) row[m * LD] += static_cast<float>(__dmul_rn(gph, sigs[m]));
@@ -1157,7 +1174,7 @@ __global__ void __launch_bounds__(NW == 1 ? 256 : 512, NW == 1 ? 2 : 1) warp_ker
 template <int NW, int NQW, bool ENERGY, bool F32>
 int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
-    constexpr int NQ = NW == 1 ? NQW : 1, max_teams = (NW == 1 ? 8 : 16) / NW;
+    constexpr int NQ = NW == 1 ? NQW : 1, max_teams = 4;
     auto layout = [&](bool slim) {
         return warp_layout(a.nv.N, a.nv.nr, a.nv.energy, F32 ? 1 : 0, a.nv.bytes_warp,
                            !F32 || a.o.scheme == KT_SCHEME_TRBDF2, a.nv.nin_max, a.nv.cvpoly, slim);
@@ -1169,9 +1186,9 @@ int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
     int smem_optin = 0, nsm = 0;
     cudaDeviceGetAttribute(&smem_optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    if (L.base + L.warp_bytes > smem_optin) L = layout(true);
+    if (L.base + L.warp_bytes > smem_optin || !a.jac) L = layout(true);
     const long long per_sm = (a.ncells + nsm - 1) / nsm;
-    int teams = c.block_warps > 0 ? c.block_warps / NW : (NW == 1 ? 4 : max_teams);
+    int teams = c.block_warps > 0 ? c.block_warps / NW : max_teams;
     if (c.block_warps <= 0 && teams > per_sm) teams = static_cast<int>(per_sm);
     if (teams > max_teams) teams = max_teams;
     if (teams < 1) teams = 1;
@@ -1198,9 +1215,10 @@ int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 
 // Dispatch over the compile-time options for one form of the iteration matrix.  Up to 32
 // unknowns one warp holds a row per lane and four would mostly wait for each other
-// (32 species, dt 1e8 s, one | four warps: 300 cells 163 | 159 ms, 2,049 cells 134 | 189,
-// 8,192 cells 207 | 475); beyond, the team is faster at every size (65 unknowns, dt 1e-9 s:
-// 1,024 cells 546 | 291 ms; 8,192 cells at 1e-10 s 615 | 405).
+// (32 species, dt 1e8 s, one | four warps, before the Jacobian program: 300 cells
+// 163 | 159 ms, 2,049 cells 134 | 189, 8,192 cells 207 | 475); beyond, the team is faster at
+// every size (65 unknowns, dt 1e-9 s: 1,024 cells 546 | 291 ms, with the program 251; 8,192
+// cells at 1e-10 s 615 | 405).
 template <bool F32, bool ENERGY>
 int launch_warp_size(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {

@@ -1,5 +1,7 @@
 """Per-lane programs of the kernels that give a cell several lanes (csrc/kt_coop_tables.cu).
 
+The larger networks' Jacobian program is laid out by the same file and replayed too.
+
 Replayed here on random rates for random networks (repeated species, one to three
 reactants, up to three products, with and without temperature): every row of f and every
 entry of I - h J must come out bit for bit as the reaction-by-reaction loop of the
@@ -34,6 +36,16 @@ extern "C" int probe(int N, int ns, int nr, int energy, const int *nin, const in
     std::memcpy(bytes, b.data(), b.size());
     return static_cast<int>(b.size());
 }
+extern "C" int team(int ns, int nr, int energy, const int *nin, const int *in, const int *rp, const int *re, int LD, int T,
+                    unsigned *prog, int cap)
+{
+    std::vector<unsigned> p;
+    const int steps = kt::team_jacobian(ns, nr, energy, nin, reinterpret_cast<const int(*)[3]>(in),
+                                        std::vector<int>(rp, rp + ns + 1), std::vector<int>(re, re + rp[ns]), LD, T, &p);
+    if (static_cast<int>(p.size()) > cap) return -2;
+    std::memcpy(prog, p.data(), 4 * p.size());
+    return steps ? steps << 16 | static_cast<int>(p.size()) / T : 0;
+}
 """
 
 
@@ -47,7 +59,7 @@ def probe(tmp_path_factory):
     src.write_text(PROBE)
     subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, str(src), "-o", str(so)], check=True,
                    capture_output=True)
-    return ctypes.CDLL(str(so)).probe
+    return ctypes.CDLL(str(so))
 
 
 def _network(rng, ns, nr):
@@ -69,7 +81,7 @@ def test_programs_replay_the_reaction_loop(probe, N, energy, nr, G, fp32):
     pin, pout, dH = pad(ins), pad(outs), rng.standard_normal(nr)
     tab, buf = np.zeros(9, ity), np.zeros(1 << 20, np.uint8)
     p = lambda a: ctypes.c_void_p(a.ctypes.data)
-    size = probe(N, ns, nr, energy, p(nin), p(nout), p(pin), p(pout), p(dH), fp32, G, p(tab), p(buf), buf.size)
+    size = probe.probe(N, ns, nr, energy, p(nin), p(nout), p(pin), p(pout), p(dH), fp32, G, p(tab), p(buf), buf.size)
     assert size > 0 and size % 16 == 0
     n_row, n_jac, off_row, off_jac, off_to, off_coef, nin_max, NM, LD = (int(v) for v in tab)
     assert nin_max == nin.max()
@@ -127,4 +139,57 @@ def test_networks_beyond_the_programs_are_left_to_the_lane_kernels(probe):
     one, sp, dH = np.ones(nr, np.int32), np.zeros((nr, 3), np.int32), np.zeros(nr)
     p = lambda a: ctypes.c_void_p(a.ctypes.data)
     for N, n in ((4, 401), (17, 10), (4, 0)):
-        assert probe(N, N, n, 0, p(one), p(one), p(sp), p(sp), p(dH), 0, 8, p(tab), p(buf), buf.size) == -1
+        assert probe.probe(N, N, n, 0, p(one), p(one), p(sp), p(sp), p(dH), 0, 8, p(tab), p(buf), buf.size) == -1
+
+
+@pytest.mark.parametrize("ns,energy,nr,LD,T", [(1, 0, 1, 4, 32), (16, 1, 75, 20, 32), (31, 1, 400, 36, 32), (32, 0, 90, 36, 32),
+                                               (33, 1, 500, 36, 128), (95, 1, 64, 100, 128)])
+def test_team_program_replays_the_row_lists(probe, ns, energy, nr, LD, T):
+    rng = np.random.default_rng(ns + nr)
+    N = ns + energy
+    ins, outs = _network(rng, ns, nr)
+    nin_max = max(map(len, ins))
+    lists = [[] for _ in range(ns)]
+    for r in range(nr):
+        for i in ins[r]:
+            lists[i].append(r << 8 | 0xff)
+        for o in outs[r]:
+            lists[o].append(r << 8 | 1)
+    ity = np.int32
+    nin, pin = np.array([len(i) for i in ins], ity), np.array([(i + [-1] * 3)[:3] for i in ins], ity)
+    rp, re = np.cumsum([0] + [len(l) for l in lists]).astype(ity), np.array(sum(lists, []) + [0], ity)
+    prog = np.zeros(1 << 18, np.uint32)
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    got = probe.team(ns, nr, energy, p(nin), p(pin), p(rp), p(re), LD, T, p(prog), prog.size)
+    assert got > 0
+    steps, total = got >> 16, got & 0xffff
+    assert steps % 8 == 0 and total == steps + 8
+    prog = prog[:total * T].reshape(total, T)
+    zero = nr * (nin_max + energy)
+    D = np.append(rng.standard_normal(zero), 0.0).astype(np.float32)
+    J = np.zeros((ns, N), np.float32)     # one list entry after the other
+    for s in range(ns):
+        for ent in lists[s]:
+            r, sg = ent >> 8, np.float32(-1 if ent & 0x80 else 1)
+            for c, col in list(enumerate(ins[r])) + ([(nin_max, ns)] if energy else []):
+                J[s, col] += sg * D[c * nr + r]
+    gotJ, seen = np.full((ns, N), np.nan, np.float32), 0
+    for t in range(T):
+        v = np.float32(0)
+        for u in prog[:steps, t].tolist():
+            d = D[u & 0x3fff]
+            v = np.float32(v + (-d if u >> 31 else d))
+            if u >> 28 & 1:
+                at = u >> 14 & 0x3fff
+                gotJ[at % LD, at // LD] = v
+                v, seen = np.float32(0), seen + 1
+    assert seen == ns * N and np.array_equal(gotJ, J)
+    assert np.all(prog[steps:] == zero)
+
+
+def test_team_program_is_left_out_beyond_its_indices(probe):
+    nr = 8200     # 2 partials each: more than 14 bits hold
+    one, sp, prog = np.ones(nr, np.int32), np.zeros((nr, 3), np.int32), np.zeros(1, np.uint32)
+    rp, re = np.zeros(3, np.int32), np.zeros(1, np.int32)
+    p = lambda a: ctypes.c_void_p(a.ctypes.data)
+    assert probe.team(2, nr, 1, p(one), p(sp), p(rp), p(re), 4, 32, p(prog), 1) == 0
