@@ -128,7 +128,8 @@ typedef struct {
     int cells_per_warp;      /* 32: the small-network kernels (<= 16 unknowns), one cell
                                 per lane or, where that is faster, per group of lanes
                                 (the same results bit for bit); 1: the large-network
-                                kernels, a cell per warp (<= 96 unknowns); 0: automatic (0) */
+                                kernels, a cell per team of one or four
+                                warps (<= 96 unknowns); 0: automatic (0) */
     int schedule;            /* kt_integrate on a state with persistent = 1: 1 hands
                                 out the cells with the most Newton iterations in the
                                 previous call first (the state's n_newton counters;
@@ -229,8 +230,8 @@ KT_API int kt_integrate_ptrs(const kt_network *net, int64_t ncells, const double
                       void *scratch, void *cuda_stream);
 
 /* Launch-configuration search (warps per block, persistent queue or one pass; the
- * kernel family is base->cells_per_warp, or by size when 0: one cell per lane up to
- * 16 unknowns, else one per warp) on a caller-supplied sample of cells in device
+ * kernel family is base->cells_per_warp, or by size when 0: the small-network kernels up
+ * to 16 unknowns, else the large-network ones) on a caller-supplied sample of cells in device
  * buffers: each candidate integrates the sample once untimed and once timed with
  * CUDA events on stream; *best receives base with the fastest configuration and
  * *best_seconds its time.  Same buffer rules as kt_integrate_ptrs; synchronises. */
@@ -248,7 +249,7 @@ KT_API int kt_autotune(const kt_network *net, int64_t ncells, const double *y_in
  * flux sigma_r when path = 0), with the exact Jacobian of tau's dependence on every
  * absorber.  rho (may be NULL: 1) also selects the cell's slice of the network's rate
  * tables.  Same buffer rules as kt_integrate_ptrs.  Networks with tabulated or photo
- * rates run in the warp-per-cell kernels (cells_per_warp 0 or 1). */
+ * rates run in the large-network kernels (cells_per_warp 0 or 1). */
 KT_API int kt_integrate_rad(const kt_network *net, int64_t ncells, const double *y_in,
                             const double *T_in, const double *rho, const double *flux,
                             const double *path, double dt, const kt_options *opts, double *y_out,
