@@ -53,6 +53,8 @@ struct AdvArgs {
 // dx / 2 times the slope of the modified van Leer limiter from the forward and backward
 // differences a and b: min(a b / (a + b), b / 2) in magnitude (the first when |a| <= |b|),
 // zero at extrema; the uniform-grid geometric factor 2c/(c+d) is 1.
+// 1/s from the hardware's seed r by the geometric series of 1/(1 - e), e = 1 - s r, cut after
+// e^2: the third-order (Chebyshev) iteration for a reciprocal.
 __device__ __forceinline__ double half_slope(double a, double b)
 {
     const double s = a + b;
