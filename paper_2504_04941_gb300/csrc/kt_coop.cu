@@ -27,12 +27,12 @@ int coop_group(const LaunchArgs &a, const LaunchCfg &c)
     if (cudaGetDevice(&dev) != cudaSuccess) return 0;
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
     const long long per = a.ncells / (4LL * nsm);   // cells per scheduler
-    const int N = a.nv.N;
-    const bool en = a.nv.energy != 0;
-    if (!en && per >= 16) return 0;
-    if (N == 11 && en) return per < 10 ? 32 : (per < 54 ? 16 : 8);
-    if (N == 3 && !en) return 4;
-    return f32 ? 0 : 16;
+    if (!a.nv.energy && per >= 16) return 0;
+    switch (coop_nm(a.nv.N, a.nv.energy)) {
+    case 3: return 4;
+    case 11: return per < 10 ? 32 : (per < 54 ? 16 : 8);
+    default: return f32 ? 0 : 16;
+    }
 }
 
 bool coop_fits(const LaunchArgs &a, const LaunchCfg &c)
@@ -47,10 +47,11 @@ bool coop_fits(const LaunchArgs &a, const LaunchCfg &c)
 
 int launch_coop(const LaunchArgs &a, const LaunchCfg &c, void *stream)
 {
-    if (a.nv.N == 3 && !a.nv.energy) return launch_coop_n3(a, c, stream);
-    if (a.nv.N == 11 && a.nv.energy)
-        return c.form == KT_FORM_FP32LU ? launch_coop_n11_f32(a, c, stream) : launch_coop_n11_f64(a, c, stream);
-    return launch_coop_any_f64(a, c, stream);
+    switch (coop_nm(a.nv.N, a.nv.energy)) {
+    case 3: return launch_coop_n3(a, c, stream);
+    case 11: return c.form == KT_FORM_FP32LU ? launch_coop_n11_f32(a, c, stream) : launch_coop_n11_f64(a, c, stream);
+    default: return launch_coop_any_f64(a, c, stream);
+    }
 }
 
 }  // namespace kt

@@ -883,8 +883,9 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
 #pragma unroll
                 for (int i = 2; i < NM; ++i) s2 = fma(fs[i], fs[i], s2);
             } else {
-                s2 = 0.0;
-                for (int i = 0; i < N; ++i) s2 = fma(fs[i], fs[i], s2);
+                const bool fixed = lane_fixed(N);
+                s2 = fixed ? fma(fs[0], fs[0], __dmul_rn(fs[1], fs[1])) : 0.0;
+                for (int i = fixed ? 2 : 0; i < N; ++i) s2 = fma(fs[i], fs[i], s2);
             }
             // s2 / N rounded once: quotient by the reciprocal of the small integer N, then one
             // correction step (Markstein 1990: correctly rounded while nothing under- or
@@ -941,6 +942,8 @@ __global__ void __launch_bounds__(kCoopMaxWarps * 32, 3) coop_kernel(const Launc
 template <int NM, int G, bool ENERGY, bool F32>
 int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
+    // (programs laid out for another size class would place the matrix by another row stride)
+    if (coop_nm(a.nv.N, a.nv.energy) != NM || a.coop_tab.ld != coop_ld(NM)) return cudaErrorInvalidConfiguration;
     CoopLayout L = coop_layout(a.nv.N, a.nv.nr, a.nv.energy, F32 ? 1 : 0, a.nv.bytes, a.nv.cvpoly, a.coop_tab);
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);

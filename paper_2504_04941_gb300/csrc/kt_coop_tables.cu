@@ -58,7 +58,7 @@ bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *n
                  std::vector<unsigned char> *bytes)
 {
     if (N > kLaneMaxN || nr < 1 || nr > kCoopMaxReactions) return false;
-    const int NM = coop_nm(N), NC = (NM + G - 1) / G, LD = coop_ld(NM);
+    const int NM = coop_nm(N, energy), NC = (NM + G - 1) / G, LD = coop_ld(NM);
     const unsigned rb = fp32 ? 4 : 8;   // bytes of a partial derivative
     std::vector<Terms> rows(N), ent(static_cast<size_t>(N) * N);
     int nin_max = 1;
@@ -96,6 +96,7 @@ bool coop_tables(int N, int ns, int nr, int energy, const int *nin, const int *n
     std::vector<unsigned> rp, jp;
     *tab = CoopTab{};
     tab->nin_max = nin_max;
+    tab->ld = LD;
     tab->n_row = pack(rows, row_lane, G, pad_row, &rp);
     tab->n_jac = pack(ent, ent_lane, G, 0u, &jp);
     std::vector<std::vector<unsigned char>> to(G);

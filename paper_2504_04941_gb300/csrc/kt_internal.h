@@ -88,9 +88,17 @@ constexpr unsigned kCoopEnd = 1u << 15;     // last term of a row or entry
 constexpr int kCoopConst = 4;               // 0, 1, -1 before the partials
 constexpr int kCoopMaxReactions = 400;    // offsets stay within 14 bits (5 kinds x 8 bytes)
 constexpr int kCoopPad = 2;                 // padding steps after each program (prefetch)
-// Compile-time size classes (3, 11, any) and row stride of the cell's matrix: rows start on
-// 16 bytes so the solve reads four FP32 factors at a time.
-constexpr int coop_nm(int N) { return N == 3 ? 3 : (N == 11 ? 11 : kLaneMaxN); }
+// Compile-time size classes (3 isothermal unknowns, 11 with temperature, any other), the one
+// place that the programs, the cell's layout and the choice of the kernel take them from, and
+// row stride of the cell's matrix: rows start on 16 bytes so the solve reads four FP32 factors
+// at a time.
+constexpr int coop_nm(int N, int energy)
+{
+    return N == 3 && !energy ? 3 : (N == 11 && energy ? 11 : kLaneMaxN);
+}
+// Sizes that the lane-per-cell kernels are compiled for, with and without temperature.
+constexpr bool lane_fixed(int N) { return N == 3 || N == 11; }
+constexpr int coop_nm(int N) { return coop_nm(N, N == 11); }   // a fixed size's own energy setting
 constexpr int coop_ld(int NM) { return (NM + 3) & ~3; }
 constexpr int kCoopMaxWarps = 4;
 
@@ -107,6 +115,7 @@ struct CoopTab {
     int off_to, off_coef;  // matrix places uint8 [k][G] of each lane's k-th entry; row
                            // coefficients, double: 0, 1, -1, -dH_r
     int nin_max;           // largest number of reactants
+    int ld;                // row stride of the matrix places (coop_ld of the size class)
     int bytes;             // multiple of 16
 };
 
@@ -252,9 +261,9 @@ inline CoopLayout coop_layout(int N, int nr, int energy, int fp32, int blob_byte
     L.off_K = energy ? 0 : take(nr * 8);
     L.off_CV = cvpoly ? take(10 * 8) : 0;
     L.off_P = take((kCoopConst + nr * (tab.nin_max + (energy ? 2 : 0))) * r);
-    L.off_M = take(N * coop_ld(coop_nm(N)) * r);
+    L.off_M = take(N * tab.ld * r);
     L.off_V = take(N * r);
-    L.off_X = take(coop_ld(coop_nm(N)) * r);
+    L.off_X = take(tab.ld * r);
     L.cell_bytes = ((o / 16) | 1) * 16;
     return L;
 }
