@@ -63,13 +63,16 @@ __device__ __forceinline__ double half_slope(double a, double b)
     double e = fma(-s, r, 1.0);
     e = fma(e, e, e);
     r = fma(r, e, r);
-    const double q = (a * r) * b;
-    const long long m = 0x7fffffffffffffffLL, inf = 0x7ff0000000000000LL;
+    double q = (a * r) * b;
+    const long long m = 0x7fffffffffffffffLL, inf = 0x7ff0000000000000LL, bit = 1LL << 52;
     const long long ba = __double_as_longlong(a), bb = __double_as_longlong(b), ia = ba & m, ib = bb & m;
-    const double half = __longlong_as_double(bb - (1LL << 52));   // b / 2 (b is normal where it is used)
+    // b / 2: one less in the exponent; below 2^-1021, where a double is the integer of its bits
+    // times 2^-1074, half of that integer (ties to even)
+    const double half = __longlong_as_double(ib >= 2 * bit ? bb - bit : (bb & ~m) | ((ib + ((ib >> 1) & 1)) >> 1));
     // zero: signs differ, a zero or a NaN, or so small (2^-959) that a b underflows
-    const bool zero = (ba ^ bb) < 0 || ia == 0 || ib == 0 || ia > inf || ib > inf ||
-                      (__double_as_longlong(s) & m) < (64LL << 52);
+    const long long is = __double_as_longlong(s) & m;
+    if (is >= 2045 * bit) q = a / s * b;   // the seed of 1/s would be subnormal: 0
+    const bool zero = (ba ^ bb) < 0 || ia == 0 || ib == 0 || ia > inf || ib > inf || is < 64 * bit;
     return zero ? 0.0 : (ia <= ib || ia == inf ? q : half);
 }
 
