@@ -92,7 +92,9 @@ __global__ void __launch_bounds__(kAdvWarps * 32) advect_kernel(const __grid_con
     const long long j0 = wrap(c0), j1 = wrap(c0 + 1), row = line * L, stride = p.nlines * L;
     const bool pair = p.vec && j1 == j0 + 1 && (j0 & 1) == 0;   // one 16-byte access
     const double inv0 = 1.0 / p.rho[row + j0], inv1 = 1.0 / p.rho[row + j1];
-    const double m0 = p.mflux[row + j0] * p.dtdx, m1 = p.mflux[row + j1] * p.dtdx;
+    // (the flux's own sign decides the upwind side: dt/dx may be negative)
+    const double g0 = p.mflux[row + j0], g1 = p.mflux[row + j1], m0 = g0 * p.dtdx, m1 = g1 * p.dtdx;
+    const bool up0 = g0 > 0.0, up1 = g1 > 0.0;
     auto load = [&](const double *a, int s) {
         const double *q = a + s * stride + row;
         if (pair) return *reinterpret_cast<const double2 *>(q + j0);
@@ -134,8 +136,8 @@ __global__ void __launch_bounds__(kAdvWarps * 32) advect_kernel(const __grid_con
         const double x0 = n.x * inv0, x1 = n.y * inv1;
         const double xp = __shfl_up_sync(0xffffffffu, x1, 1, W), hp = __shfl_up_sync(0xffffffffu, h.y, 1, W);
         // upwind states at the lower interfaces of the two cells, then dt/dx times the fluxes
-        const double f0 = ((m0 > 0.0 ? xp : x0) + (m0 > 0.0 ? hp : -h.x)) * m0;
-        const double f1 = ((m1 > 0.0 ? x0 : x1) + (m1 > 0.0 ? h.x : -h.y)) * m1;
+        const double f0 = ((up0 ? xp : x0) + (up0 ? hp : -h.x)) * m0;
+        const double f1 = ((up1 ? x0 : x1) + (up1 ? h.x : -h.y)) * m1;
         const double f2 = __shfl_down_sync(0xffffffffu, f0, 1, W);
         double v0 = n.x + (f0 - f1), v1 = n.y + (f1 - f2);
         if (p.n_base) {

@@ -49,3 +49,14 @@ def test_large_abundances(kt):  # noqa: F811
     # the same with everything scaled by 2^-40, where nothing is near the range's end
     ref = A.advect_step(n * 2.0 ** -40, rho, flux, 0.3, 0.37, None)
     assert np.all(np.abs(got * 2.0 ** -40 - ref) <= 1e-12 * 1e308 * 2.0 ** -40)
+
+
+@pytest.mark.parametrize("project", [False, True])
+@pytest.mark.parametrize("dtdx", [-0.3, 0.0, 0.3])
+def test_upwind_side_follows_the_flux_for_either_sign_of_dtdx(kt, dtdx, project):  # noqa: F811
+    netw = _network(5, 2, 4)
+    rng = np.random.default_rng(8)
+    n, rho, flux = rng.uniform(0.1, 1.0, (5, 4, 33)), rng.uniform(0.5, 2.0, (4, 33)), rng.uniform(-1.0, 1.0, (4, 33))
+    ref = A.advect_step(n, rho, flux, dtdx, 0.37, A.element_projector(netw.counts) if project else None)
+    got = _sweep(kt, netw, n, rho, flux, dtdx, project)
+    assert np.all(np.abs(got - ref) <= 1e-12 * (n.max() + 0.6 * (n / rho[None]).max()))
