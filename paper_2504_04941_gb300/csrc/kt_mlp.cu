@@ -3,7 +3,7 @@
 // Parameters live twice: FP32 master weights (Adam state beside them) and the packed
 // BF16 block of kt_mlp.cuh that the tensor-core kernels read.  One training step:
 //   train_tile    one block per 64 samples, a warp per 16: the parameters are staged in
-//                 shared memory by one bulk copy, then forward, MSE loss gradient and backward
+//                 shared memory by 16-byte asynchronous copies, then forward, MSE loss gradient and backward
 //                 (dz_l = (dz_{l+1} W_{l+1}) * s_l) with activations h_l and SiLU
 //                 derivatives s_l / dz_l kept in shared memory as BF16, then this tile's
 //                 dW_l = dz_l^T h_{l-1} and db_l into the block's own FP32 partial;
@@ -27,7 +27,7 @@
 
 #include "kt_internal.h"
 #include "kt_mlp.cuh"
-#include "kt_tma.cuh"
+#include "kt_tma.cuh"   // smem_u32
 
 namespace kt {
 namespace {
@@ -51,6 +51,19 @@ __device__ __forceinline__ float silu_grad_f(float z)
 {
     const float s = 1.0f / (1.0f + __expf(-z));
     return s * (1.0f + z * (1.0f - s));
+}
+
+// The packed parameters to shared memory, 16 bytes per copy.  The wait is the hardware's own and
+// cannot give up, so no launch leaves its outputs unwritten.  Every thread of the block calls it.
+__device__ __forceinline__ void stage_params(unsigned char *sm, const unsigned char *P)
+{
+    static_assert(MlpLayout::BYTES % 16 == 0, "16-byte copies");
+    for (int i = threadIdx.x * 16; i < MlpLayout::BYTES; i += blockDim.x * 16)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(sm + i)),
+                     "l"(__cvta_generic_to_global(P + i))
+                     : "memory");
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
 }
 
 // 8x8 BF16 blocks of shared memory, transposed (lane 8 i + r gives row r of block i).
@@ -101,8 +114,7 @@ constexpr int kMaxPartials = 512;         // blocks of one launch; each loops ov
 // Shared memory of train_tile (bytes): the packed parameters, the activations h0 .. h3 and
 // the SiLU derivatives s1 .. s3, overwritten by dz1 .. dz3, and dz4; rows padded by 16 bytes.
 struct TileLayout {
-    static constexpr int BAR = (MlpLayout::BYTES + 15) & ~15;
-    static constexpr int H0 = BAR + 16;
+    static constexpr int H0 = MlpLayout::BYTES;
     static constexpr int H1 = H0 + kTile * kMlpKP1 * 2;
     static constexpr int HB = kTile * kMlpKP * 2;
     static constexpr int D1 = H1 + 3 * HB;
@@ -116,15 +128,13 @@ struct TrainArgs {
     const float *X, *Tg;             // [B][16], [B][16]
     float *part;                     // [blocks][Master::N]
     double *loss;                    // [blocks]
-    int *err;                        // device error word
     int B, nout;
 };
 
 __global__ void __launch_bounds__(kTrainWarps * 32, 1) train_tile(const TrainArgs a)
 {
     extern __shared__ __align__(16) unsigned char sm[];
-    if (!stage_table(sm, a.P, MlpLayout::BYTES, reinterpret_cast<uint64_t *>(sm + TileLayout::BAR), a.err, kDevErrTma))
-        return;
+    stage_params(sm, a.P);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, g = lane >> 2, t = lane & 3;
     auto rows = [&](int off) { return reinterpret_cast<__nv_bfloat16 *>(sm + off); };
     __nv_bfloat16 *H0 = rows(TileLayout::H0), *D4 = rows(TileLayout::D4);
@@ -360,10 +370,10 @@ __global__ void adam(float *p, float *m, float *v, const float *g, unsigned char
 // batch inference: X [n][16] -> out [n][16], one warp per 16 rows, the parameters staged in
 // shared memory once per block (read from global memory fragment by fragment a call took
 // 19.5 us at any size up to 16,384 rows)
-__global__ void __launch_bounds__(128) infer(const unsigned char *P, const float *X, float *out, long long n, int *err)
+__global__ void __launch_bounds__(128) infer(const unsigned char *P, const float *X, float *out, long long n)
 {
     extern __shared__ __align__(16) unsigned char sm[];
-    if (!stage_table(sm, P, MlpLayout::BYTES, reinterpret_cast<uint64_t *>(sm + TileLayout::BAR), err, kDevErrTma)) return;
+    stage_params(sm, P);
     const int lane = threadIdx.x & 31;
     const int g = lane >> 2, t = lane & 3;
     for (long long m0 = ((static_cast<long long>(blockIdx.x) * blockDim.x + threadIdx.x) >> 5) * 16; m0 < n;
@@ -426,7 +436,6 @@ struct kt_mlp {
     float *part = nullptr;                        // their gradient partials [cap][Master::N]
     double *lpart = nullptr;                      // and losses [cap]
     double *loss = nullptr;                       // the batch's loss
-    int *err = nullptr;                           // device error word
     std::vector<float> norm = std::vector<float>(kt::MlpLayout::NNORM, 0.0f);
 
     ~kt_mlp()
@@ -439,7 +448,6 @@ struct kt_mlp {
         cudaFree(part);
         cudaFree(lpart);
         cudaFree(loss);
-        cudaFree(err);
     }
 
     int ensure(int blocks)
@@ -524,8 +532,6 @@ int kt_mlp_create(int n_in, int n_out, unsigned long long seed, kt_mlp **out)
     if (e == cudaSuccess) e = cudaMalloc(&m->v, kt::Master::N * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->g, kt::Master::N * 4);
     if (e == cudaSuccess) e = cudaMalloc(&m->loss, sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&m->err, sizeof(int));
-    if (e == cudaSuccess) e = cudaMemset(m->err, 0, sizeof(int));
     if (e == cudaSuccess) e = cudaMemset(m->m, 0, kt::Master::N * 4);
     if (e == cudaSuccess) e = cudaMemset(m->v, 0, kt::Master::N * 4);
     if (e != cudaSuccess) {
@@ -594,25 +600,11 @@ static int fwd_bwd(kt_mlp *m, const float *X, const float *T, int B, cudaStream_
     if (rc) return rc;
     cudaError_t e = cudaFuncSetAttribute(kt::train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, kt::TileLayout::BYTES);
     if (e != cudaSuccess) return mcuda(e, "kt_mlp: train kernel attributes");
-    const kt::TrainArgs a{m->P, X, T, m->part, m->lpart, m->err, B, m->nout};
+    const kt::TrainArgs a{m->P, X, T, m->part, m->lpart, B, m->nout};
     kt::train_tile<<<blocks, kt::kTrainWarps * 32, kt::TileLayout::BYTES, s>>>(a);
     kt::reduce_grads<<<(kt::Master::N / 4 + 127) / 128, 128, 0, s>>>(m->part, m->lpart, blocks, m->g, m->loss);
     e = cudaGetLastError();
     return e == cudaSuccess ? KT_OK : mcuda(e, "kt_mlp: train kernels");
-}
-
-// A device wait that gave up (the stream is synchronised by the caller).
-static int check_err(kt_mlp *m, cudaStream_t s)
-{
-    int h = 0;
-    cudaError_t e = cudaMemcpyAsync(&h, m->err, sizeof h, cudaMemcpyDeviceToHost, s);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
-    if (e != cudaSuccess) return mcuda(e, "kt_mlp: error word");
-    if (h) {
-        cudaMemsetAsync(m->err, 0, sizeof h, s);
-        return mfail(KT_ETIMEOUT, "device: a bounded wait for the parameter copy gave up");
-    }
-    return KT_OK;
 }
 
 int kt_mlp_train_step(kt_mlp *m, const float *X, const float *T, int B, float lr, double *loss, void *stream)
@@ -627,8 +619,8 @@ int kt_mlp_train_step(kt_mlp *m, const float *X, const float *T, int B, float lr
     if (e != cudaSuccess) return mcuda(e, "kt_mlp: adam");
     if (loss) {
         e = cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, s);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(s);
         if (e != cudaSuccess) return mcuda(e, "kt_mlp: loss readback");
-        return check_err(m, s);
     }
     return KT_OK;
 }
@@ -641,7 +633,8 @@ int kt_mlp_gradients(kt_mlp *m, const float *X, const float *T, int B, float *gr
     if (rc) return rc;
     cudaError_t e = cudaMemcpyAsync(grads, m->g, kt::Master::N * 4, cudaMemcpyDeviceToHost, s);
     if (e == cudaSuccess && loss) e = cudaMemcpyAsync(loss, m->loss, sizeof(double), cudaMemcpyDeviceToHost, s);
-    return e == cudaSuccess ? check_err(m, s) : mcuda(e, "kt_mlp_gradients");
+    if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+    return e == cudaSuccess ? KT_OK : mcuda(e, "kt_mlp_gradients");
 }
 
 int kt_mlp_forward(const kt_mlp *m, const float *X, float *out, int64_t n, void *stream)
@@ -654,11 +647,11 @@ int kt_mlp_forward(const kt_mlp *m, const float *X, float *out, int64_t n, void 
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    const int smem = kt::TileLayout::BAR + 16;
+    const int smem = kt::MlpLayout::BYTES;
     cudaError_t e = cudaFuncSetAttribute(kt::infer, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return mcuda(e, "kt_mlp_forward");
     kt::infer<<<static_cast<unsigned>(blocks < 2LL * nsm ? blocks : 2LL * nsm), 128, smem,
-                static_cast<cudaStream_t>(stream)>>>(m->P, X, out, n, m->err);
+                static_cast<cudaStream_t>(stream)>>>(m->P, X, out, n);
     e = cudaGetLastError();
     return e == cudaSuccess ? KT_OK : mcuda(e, "kt_mlp_forward");
 }
