@@ -38,7 +38,24 @@ struct RayArgs {
 // 2^(j/256) and what its rounding to double leaves (kt_exp.cuh).
 struct RayExpTable {
     double hi[kExpTable], lo[kExpTable];
+
+    RayExpTable()
+    {
+        for (int j = 0; j < kExpTable; ++j) {
+            hi[j] = exp2_table(j);
+            lo[j] = static_cast<double>(std::exp2(static_cast<long double>(j) / static_cast<long double>(kExpTable)) -
+                                        static_cast<long double>(hi[j]));
+        }
+    }
 };
+
+// Formed by the first call of the process: 512 long double powers take an Arm host, where that
+// type is software, about 250 us (a trace of 64 rays through 4^3 cells: 78 us).
+const RayExpTable &ray_exp_table()
+{
+    static const RayExpTable table;
+    return table;
+}
 
 // e^-tau and 1 - e^-tau for 0 <= tau < 700: -tau = (256 m + j) ln2/256 + r, e^-tau =
 // S (1 + p) with S = 2^(j/256) 2^m and p = e^r - 1 (kt_exp.cuh); 1 - e^-tau is summed as
@@ -210,12 +227,7 @@ extern "C" KT_API int kt_raytrace(int nx, int ny, int nz, double hx, double hy, 
         return KT_EINVAL;
     }
     kt::RayArgs a{nx, ny, nz, nbins, hx, hy, hz, dt, nrays, kappa, origins, dirs, n0, feff, absorbed, escaped};
-    kt::RayExpTable tab;
-    for (int j = 0; j < kt::kExpTable; ++j) {
-        const long double v = std::exp2(static_cast<long double>(j) / static_cast<long double>(kt::kExpTable));
-        tab.hi[j] = kt::exp2_table(j);
-        tab.lo[j] = static_cast<double>(v - static_cast<long double>(tab.hi[j]));
-    }
+    const kt::RayExpTable &tab = kt::ray_exp_table();
     const int threads = 128;
     const unsigned blocks = static_cast<unsigned>((nrays + threads - 1) / threads);
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
