@@ -71,11 +71,15 @@ struct kt_network {
     std::vector<double> tab;                      // [ntab][nR][nT] ln k
     std::vector<unsigned char> blob;
     NetView view{};
-    // programs of the kernels with 4, 8, 16 or 32 lanes per cell (FP64 form, then FP32-LU):
-    // they follow the tables (view.bytes_total) in the blob; -1 where the network has none
+    // Programs of the kernels with several lanes or warps per cell, laid out by the first call
+    // that integrates (a program that only advects with the network does not pay for them) and
+    // unchanged from then on; in the device copy they follow the tables (view.bytes_total).
+    bool laid_out = false;
+    std::vector<unsigned char> prog;
+    // 4, 8, 16 or 32 lanes per cell (FP64 form, then FP32-LU): offsets in prog, -1: none
     std::array<int, 8> coop_off{{-1, -1, -1, -1, -1, -1, -1, -1}};
     std::array<kt::CoopTab, 8> coop_tab{};
-    // Jacobian program of the larger-network kernels (FP64 form, FP32-LU), also in the blob
+    // Jacobian programs of the larger-network kernels (FP64 form, FP32-LU)
     std::array<int, 2> jac_off{{-1, -1}}, jac_steps{{0, 0}}, jac_bytes{{0, 0}};
     const kt_mlp *mlp = nullptr;                  // attached learned-guess MLP (not owned)
     std::mutex mu;
@@ -92,7 +96,10 @@ struct kt_network {
         cudaSetDevice(cur);
     }
 
-    // Device copy of the blob on the current device (uploaded once per device).
+    // Lays the programs out on the first call (mu is held).
+    int lay_out();
+
+    // Device copy of the tables and programs on the current device (uploaded once per device).
     int device_blob(const unsigned char **out)
     {
         int dev = 0;
@@ -104,10 +111,14 @@ struct kt_network {
             *out = it->second;
             return KT_OK;
         }
+        const int rc = lay_out();
+        if (rc != KT_OK) return rc;
         unsigned char *p = nullptr;
-        e = cudaMalloc(&p, blob.size());
+        e = cudaMalloc(&p, blob.size() + prog.size());
         if (e != cudaSuccess) return fail(KT_ENOMEM, "cudaMalloc(network tables): %s", cudaGetErrorString(e));
         e = cudaMemcpy(p, blob.data(), blob.size(), cudaMemcpyHostToDevice);
+        if (e == cudaSuccess && !prog.empty())
+            e = cudaMemcpy(p + blob.size(), prog.data(), prog.size(), cudaMemcpyHostToDevice);
         if (e != cudaSuccess) {
             cudaFree(p);
             return cuda_fail(e, "cudaMemcpy(network tables)");
@@ -426,7 +437,7 @@ void build_blob(kt_network *n)
     }
 }
 
-// Appends the Jacobian programs of the larger-network kernels to the blob.
+// The Jacobian programs of the larger-network kernels.
 void build_team(kt_network *n)
 {
     const int N = n->view.N, T = N <= 32 ? 32 : 128;
@@ -441,16 +452,16 @@ void build_team(kt_network *n)
                                             reinterpret_cast<const int(*)[kt::kMaxSide]>(n->in.data()), rp, re, LD, T,
                                             &prog);
         if (!steps) continue;
-        n->jac_off[f] = static_cast<int>(n->blob.size());
+        n->jac_off[f] = static_cast<int>(n->prog.size());
         n->jac_steps[f] = steps;
         n->jac_bytes[f] = static_cast<int>(4 * prog.size());
         const unsigned char *b = reinterpret_cast<const unsigned char *>(prog.data());
-        n->blob.insert(n->blob.end(), b, b + n->jac_bytes[f]);
-        n->blob.resize((n->blob.size() + 15) & ~static_cast<size_t>(15));
+        n->prog.insert(n->prog.end(), b, b + n->jac_bytes[f]);
+        n->prog.resize((n->prog.size() + 15) & ~static_cast<size_t>(15));
     }
 }
 
-// Appends the per-lane programs of every group size to the blob.
+// The per-lane programs of the group sizes that there are kernels for.
 void build_coop(kt_network *n)
 {
     if (n->ns + n->energy > kt::kLaneMaxN || n->view.special) return;
@@ -458,13 +469,14 @@ void build_coop(kt_network *n)
     std::vector<double> dH(n->nr);
     std::memcpy(dH.data(), n->blob.data() + n->view.off_dH, 8 * dH.size());
     for (int i = 0; i < 8; ++i) {
+        if (!(kt::coop_sizes(kt::coop_nm(n->view.N, n->energy), i >= 4) >> (i & 3) & 1u)) continue;
         if (!kt::coop_tables(n->view.N, n->ns, n->nr, n->energy, n->nin.data(), n->nout.data(),
                              reinterpret_cast<const int(*)[kt::kMaxSide]>(n->in.data()),
                              reinterpret_cast<const int(*)[kt::kMaxSide]>(n->out.data()), dH.data(), i >= 4,
                              4 << (i & 3), &n->coop_tab[i], &prog))
             return;
-        n->coop_off[i] = static_cast<int>(n->blob.size());
-        n->blob.insert(n->blob.end(), prog.begin(), prog.end());
+        n->coop_off[i] = static_cast<int>(n->prog.size());
+        n->prog.insert(n->prog.end(), prog.begin(), prog.end());
     }
 }
 
@@ -508,6 +520,22 @@ kt::DevOpts dev_opts(const kt_options *o)
 
 }  // namespace
 
+int kt_network::lay_out()
+{
+    if (laid_out) return KT_OK;
+    try {
+        build_coop(this);
+        build_team(this);
+    } catch (const std::bad_alloc &) {
+        prog.clear();
+        coop_off.fill(-1);
+        jac_off.fill(-1);
+        return fail(KT_ENOMEM, "network programs: out of memory");
+    }
+    laid_out = true;
+    return KT_OK;
+}
+
 extern "C" {
 
 const char *kt_last_error(void) { return g_err.c_str(); }
@@ -549,8 +577,6 @@ int kt_network_load(const char *path, kt_network **out)
         return rc;
     }
     build_blob(n);
-    build_coop(n);
-    build_team(n);
     *out = n;
     return KT_OK;
 }
@@ -671,14 +697,14 @@ int integrate_impl(const kt_network *net, int64_t ncells, const double *y_in, co
     const int grp = cpw == 32 ? kt::coop_group(a, c) : 0;
     const int gi = (grp == 4 ? 0 : (grp == 8 ? 1 : (grp == 16 ? 2 : 3))) + (opts->form == KT_FORM_FP32LU ? 4 : 0);
     if (grp && net->coop_off[gi] >= 0) {
-        a.coop = blob + net->coop_off[gi];
+        a.coop = blob + net->view.bytes_total + net->coop_off[gi];
         a.coop_tab = net->coop_tab[gi];
         a.coop_g = grp;
         if (!kt::coop_fits(a, c)) a.coop = nullptr;
     }
     const int f32 = opts->form == KT_FORM_FP32LU;
     if (cpw == 1 && net->jac_off[f32] >= 0) {
-        a.jac = reinterpret_cast<const unsigned *>(blob + net->jac_off[f32]);
+        a.jac = reinterpret_cast<const unsigned *>(blob + net->view.bytes_total + net->jac_off[f32]);
         a.jac_steps = net->jac_steps[f32];
     }
     int ce = a.coop ? kt::launch_coop(a, c, cuda_stream)
@@ -766,8 +792,14 @@ int kt::prepare_launch(const kt_network *net, int64_t ncells, const double *y_in
     const int f32 = opts->form == KT_FORM_FP32LU;
     *host_jac = nullptr;
     *jac_bytes = 0;
+    if (cpw == 1) {
+        kt_network *mn = const_cast<kt_network *>(net);
+        std::lock_guard<std::mutex> lk(mn->mu);
+        rc = mn->lay_out();
+        if (rc) return rc;
+    }
     if (cpw == 1 && net->jac_off[f32] >= 0) {
-        *host_jac = net->blob.data() + net->jac_off[f32];
+        *host_jac = net->prog.data() + net->jac_off[f32];
         *jac_bytes = net->jac_bytes[f32];
         a->jac_steps = net->jac_steps[f32];
     }

@@ -100,6 +100,11 @@ constexpr int coop_nm(int N, int energy)
 constexpr bool lane_fixed(int N) { return N == 3 || N == 11; }
 constexpr int coop_nm(int N) { return coop_nm(N, N == 11); }   // a fixed size's own energy setting
 constexpr int coop_ld(int NM) { return (NM + 3) & ~3; }
+// Lanes per cell for which a size class and form have kernels, of 4, 8, 16 and 32 (bits 0..3).
+constexpr unsigned coop_sizes(int NM, bool fp32)
+{
+    return NM == 3 ? 1u : (NM == 11 ? 14u : (fp32 ? 0u : 4u));
+}
 constexpr int kCoopMaxWarps = 4;
 
 // Jacobian program of the larger-network kernels: [step][thread] terms, a term being the

@@ -38,7 +38,8 @@ PROBE = r"""
 #include "kt_coop.cu"
 #include "kt_coop_tables.cu"
 // out: lanes per cell (0: one cell per lane), size of the kernel, largest matrix place
-// written, first byte of the matrix, first byte behind it, element size, groups' fit
+// written, first byte of the matrix, first byte behind it, element size, whether the programs
+// of that many lanes are laid out
 extern "C" int route(int N, int energy, int form, int scheme, long long ncells, int nr, const int *nin, const int *in,
                      int *out)
 {
@@ -65,6 +66,7 @@ extern "C" int route(int N, int energy, int form, int scheme, long long ncells, 
     out[3] = L.off_M;
     out[4] = L.off_V;
     out[5] = f32 ? 4 : 8;
+    out[6] = kt::coop_sizes(kt::coop_nm(N, energy), f32) * 4 & a.coop_g;
     return 1;
 }
 """
@@ -100,12 +102,13 @@ def test_programs_and_kernel_agree_on_the_row_stride(probe, N, energy, form):
     p = lambda a: ctypes.c_void_p(a.ctypes.data)
     for scheme in (0, 1):
         for ncells in (1, 250, 6079, 6080, 9727, 9728, 32832, 65536, 10**6):
-            out = np.zeros(6, np.int32)
+            out = np.zeros(7, np.int32)
             got = probe.route(N, energy, form, scheme, ncells, nr, p(nin), p(pin), p(out))
             assert got >= 0
             if got == 0:
                 continue
-            NM, written, begin, end, size = (int(v) for v in out[1:])
+            NM, written, begin, end, size, laid_out = (int(v) for v in out[1:])
+            assert laid_out
             assert N <= NM
             ld = (NM + 3) & ~3                       # rows of the kernel's matrix
             assert written == (N - 1) * ld + N - 1   # the last entry lies where the kernel reads it
