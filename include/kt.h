@@ -78,7 +78,7 @@ extern "C" {
                                order.  The second stage starts from the first stage's
                                result whatever `guess` says; KT_GUESS_MLP is refused. */
 
-/* storage of the FP32-LU lane-per-cell kernels under TR-BDF2 (kt_options.lane_variant) */
+/* variant of the FP32-LU small-network kernels under TR-BDF2 (kt_options.lane_variant) */
 #define KT_LANE_AUTO 0      /* KT_LANE_LEAN where it applies */
 #define KT_LANE_JCACHE 1    /* the FP32 Jacobian is kept beside the iteration matrix (a
                                rejected attempt re-uses it) and a failed FP32 solve is
@@ -88,7 +88,9 @@ extern "C" {
                                FP32 (no Jacobian copy), the step's start state and rate
                                stay in registers, and a failed FP32 solve halves h (no
                                FP64 rescue); 27 KB per warp for 11 unknowns, so twice as
-                               many warps share an SM */
+                               many warps share an SM.  The kernels with a group of lanes
+                               per cell do the same arithmetic, result for result, and are
+                               taken for it where they are faster (cells_per_warp) */
 
 typedef struct kt_network kt_network;
 typedef struct kt_state kt_state;
@@ -122,7 +124,10 @@ typedef struct {
     int retry;               /* 1: retry failed cells once                      (1) */
     int atol_mode;           /* 0: atol absolute; 1: atol times the cell's
                                 initial total of element 0                     (0) */
-    int block_warps;         /* warps per block, 0 = automatic                   (0) */
+    int block_warps;         /* warps per block, 0 = automatic; at most 8 with one cell
+                                per lane, 4 with groups of lanes and four teams'
+                                worth in the large-network kernels (4, or 16 beyond
+                                32 unknowns): a larger value launches that many  (0) */
     int blocks_per_sm;       /* persistent grid = blocks_per_sm x SMs, 0 = automatic (0) */
     int use_graph;           /* 1: kt_integrate replays a captured CUDA graph    (0) */
     int cells_per_warp;      /* 32: the small-network kernels (<= 16 unknowns), one cell
@@ -136,7 +141,7 @@ typedef struct {
                                 zero after kt_state_create), 0 in index order.  The
                                 order changes no result, only the load balance (0) */
     int scheme;              /* KT_SCHEME_*: the one-step scheme of each sub-step      (BE) */
-    int lane_variant;        /* KT_LANE_*: storage of the FP32-LU lane-per-cell kernels
+    int lane_variant;        /* KT_LANE_*: variant of the FP32-LU small-network kernels
                                 with TR-BDF2 (3 or 11 unknowns); ignored elsewhere (AUTO) */
     int reserved[2];
 } kt_options;

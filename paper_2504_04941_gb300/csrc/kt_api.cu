@@ -440,7 +440,7 @@ void build_blob(kt_network *n)
 // The Jacobian programs of the larger-network kernels.
 void build_team(kt_network *n)
 {
-    const int N = n->view.N, T = N <= 32 ? 32 : 128;
+    const int N = n->view.N, T = 32 * kt::team_warps(n->view.N);
     if (N > kt::kWarpMaxN || n->nr < 1) return;
     std::vector<int> rp(n->ns + 1), re(n->view.nent);
     std::memcpy(rp.data(), n->blob.data() + n->view.off_rp, 4 * rp.size());
@@ -629,6 +629,19 @@ int state_schedule(kt_state *st, const kt_options *opts, cudaStream_t s, bool la
     return KT_OK;
 }
 
+// Sends the call to the kernels with several lanes per cell (a->coop) where they are the faster
+// ones and the network's programs and a warp's cells fit.
+void route_groups(const kt_network *net, const unsigned char *blob, const kt::LaunchCfg &c, kt::LaunchArgs *a)
+{
+    const int grp = c.cells_per_warp == 32 ? kt::coop_group(*a, c) : 0;
+    const int gi = (grp == 4 ? 0 : (grp == 8 ? 1 : (grp == 16 ? 2 : 3))) + (c.form == KT_FORM_FP32LU ? 4 : 0);
+    if (!grp || net->coop_off[gi] < 0) return;
+    a->coop = blob + net->view.bytes_total + net->coop_off[gi];
+    a->coop_tab = net->coop_tab[gi];
+    a->coop_g = grp;
+    if (!kt::coop_fits(*a, c)) a->coop = nullptr;
+}
+
 int integrate_impl(const kt_network *net, int64_t ncells, const double *y_in, const double *T_in,
                    const double *rho, const double *dt_cell, double dt, const kt_options *opts, double *y_out,
                    double *T_out, int32_t *status, int32_t *n_substeps, int32_t *n_newton, void *scratch,
@@ -694,14 +707,7 @@ int integrate_impl(const kt_network *net, int64_t ncells, const double *y_in, co
     a.order = opts->persistent ? order : nullptr;
     kt::LaunchCfg c{opts->form, opts->persistent, opts->block_warps, opts->blocks_per_sm, cpw, opts->lane_variant};
     a.persistent = opts->persistent != 0;
-    const int grp = cpw == 32 ? kt::coop_group(a, c) : 0;
-    const int gi = (grp == 4 ? 0 : (grp == 8 ? 1 : (grp == 16 ? 2 : 3))) + (opts->form == KT_FORM_FP32LU ? 4 : 0);
-    if (grp && net->coop_off[gi] >= 0) {
-        a.coop = blob + net->view.bytes_total + net->coop_off[gi];
-        a.coop_tab = net->coop_tab[gi];
-        a.coop_g = grp;
-        if (!kt::coop_fits(a, c)) a.coop = nullptr;
-    }
+    route_groups(net, blob, c, &a);
     const int f32 = opts->form == KT_FORM_FP32LU;
     if (cpw == 1 && net->jac_off[f32] >= 0) {
         a.jac = reinterpret_cast<const unsigned *>(blob + net->view.bytes_total + net->jac_off[f32]);
@@ -1024,6 +1030,9 @@ int kt_autotune(const kt_network *net, int64_t ncells, const double *y_in, const
     int rc = check_opts(base);
     if (rc) return rc;
     const int N = net->ns + net->energy;
+    const unsigned char *blob = nullptr;
+    rc = const_cast<kt_network *>(net)->device_blob(&blob);
+    if (rc) return rc;
     cudaStream_t s = static_cast<cudaStream_t>(cuda_stream);
     cudaEvent_t e0 = nullptr, e1 = nullptr;
     cudaError_t e = cudaEventCreate(&e0);
@@ -1031,22 +1040,30 @@ int kt_autotune(const kt_network *net, int64_t ncells, const double *y_in, const
     if (e != cudaSuccess) return cuda_fail(e, "kt_autotune: cudaEventCreate");
     double best_t = 1e300;
     kt_options cand = *base, win = *base;
-    // The kernel family follows the size unless the caller fixed it: one cell per lane
-    // when it fits (every FP64 warp instruction then serves 32 cells), else one per
-    // warp.  A short tuning sample cannot judge that choice (short integrations are
-    // latency-bound and favour one cell per warp), so only the launch shape is searched.
+    // The kernel family follows the size unless the caller fixed it: the small-network kernels
+    // (a cell per lane or per group of lanes, whichever the dispatch takes for the sample)
+    // up to 16 unknowns, else a cell per team of warps.  A short tuning sample cannot judge
+    // that choice (short integrations are latency-bound), so only the launch shape is searched.
     const int fam = base->cells_per_warp ? base->cells_per_warp : (N <= kt::kLaneMaxN ? 32 : 1);
     const int cpws[1] = {fam};
-    const int bws[4] = {1, 2, 4, 8};
-    // the FP32-LU lane kernels under TR-BDF2 come in two storage variants (kt.h KT_LANE_*)
+    // the FP32-LU kernels of these networks come in two variants under TR-BDF2 (kt.h KT_LANE_*)
     const bool two = fam == 32 && base->form == KT_FORM_FP32LU && base->scheme == KT_SCHEME_TRBDF2 &&
                      base->lane_variant == KT_LANE_AUTO;
     const int vars[2] = {two ? KT_LANE_JCACHE : base->lane_variant, KT_LANE_LEAN};
     for (int ci = 0; ci < 1; ++ci) {
         if (cpws[ci] == 32 && N > kt::kLaneMaxN) continue;
         for (int vi = 0; vi < (two ? 2 : 1); ++vi)
-        for (int per = 0; per <= 1; ++per)
-            for (int bi = 0; bi < 4; ++bi) {
+        for (int per = 0; per <= 1; ++per) {
+            // shapes that differ in the kernel this variant runs in
+            kt::LaunchArgs a{};
+            a.nv = net->view;
+            a.o = dev_opts(base);
+            a.ncells = ncells;
+            a.mlp = base->guess == KT_GUESS_MLP ? blob : nullptr;
+            route_groups(net, blob, kt::LaunchCfg{base->form, per, 0, 0, fam, vars[vi]}, &a);
+            int bws[4];
+            const int shapes = kt::block_shapes(N, fam, a.coop != nullptr, bws);
+            for (int bi = 0; bi < shapes; ++bi) {
                 cand.cells_per_warp = cpws[ci];
                 cand.lane_variant = vars[vi];
                 cand.persistent = per;
@@ -1073,6 +1090,7 @@ int kt_autotune(const kt_network *net, int64_t ncells, const double *y_in, const
                     win = cand;
                 }
             }
+        }
         if (rc) break;
     }
     cudaEventDestroy(e0);

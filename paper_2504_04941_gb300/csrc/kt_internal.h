@@ -12,6 +12,7 @@ namespace kt {
 constexpr int kMaxSide = 3;      // reactants / products per reaction
 constexpr int kMaxElements = 8;
 constexpr int kLaneMaxN = 16;    // unknowns per cell handled by the lane-per-cell kernels
+constexpr int kLaneMaxWarps = 8; // warps per block of those kernels
 constexpr int kIdxNone = 255;
 constexpr int kIdxDistinct = 0x80;   // flag in the reactant-count byte: all species differ
 constexpr int kExpTable = 256;       // entries 2^(j/256) of the table-driven exponential
@@ -106,6 +107,19 @@ constexpr unsigned coop_sizes(int NM, bool fp32)
     return NM == 3 ? 1u : (NM == 11 ? 14u : (fp32 ? 0u : 4u));
 }
 constexpr int kCoopMaxWarps = 4;
+// The larger-network kernels: warps per team (cell) and teams per block.
+constexpr int team_warps(int N) { return N <= 32 ? 1 : 4; }
+constexpr int kMaxTeams = 4;
+// Values of block_warps that launch blocks of different shapes (a larger one launches the
+// largest): warps of 32 cells (8 at most) or of groups (4), or whole teams.  Returns how many.
+inline int block_shapes(int N, int cells_per_warp, bool groups, int (&warps)[4])
+{
+    const int unit = cells_per_warp == 1 ? team_warps(N) : 1;
+    const int most = cells_per_warp == 1 ? kMaxTeams : (groups ? kCoopMaxWarps : kLaneMaxWarps);
+    int n = 0;
+    for (int k = 1; k <= most; k *= 2) warps[n++] = k * unit;
+    return n;
+}
 
 // Jacobian program of the larger-network kernels: [step][thread] terms, a term being the
 // partial's index (bits 0..13), the entry's place in the matrix (14..27, with kTermEnd) and

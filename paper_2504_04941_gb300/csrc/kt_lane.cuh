@@ -52,7 +52,7 @@ namespace kt {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kMaxWarps = 8;
+constexpr int kMaxWarps = kLaneMaxWarps;
 
 #define LI(p, e) ((p)[(e) << 5])
 // per-lane arrays with a stride of 2^SH words (FP32 arrays interleave two per lane)

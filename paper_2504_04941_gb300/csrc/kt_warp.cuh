@@ -1174,7 +1174,7 @@ __global__ void __launch_bounds__(NW == 1 ? 128 : 512, NW == 1 ? 3 : 1) warp_ker
 template <int NW, int NQW, bool ENERGY, bool F32>
 int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
-    constexpr int NQ = NW == 1 ? NQW : 1, max_teams = 4;
+    constexpr int NQ = NW == 1 ? NQW : 1, max_teams = kMaxTeams;
     auto layout = [&](bool slim) {
         return warp_layout(a.nv.N, a.nv.nr, a.nv.energy, F32 ? 1 : 0, a.nv.bytes_warp,
                            !F32 || a.o.scheme == KT_SCHEME_TRBDF2, a.nv.nin_max, a.nv.cvpoly, slim);
@@ -1222,7 +1222,7 @@ int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 template <bool F32, bool ENERGY>
 int launch_warp_size(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 {
-    return a.nv.N <= 32 ? launch_t<1, 1, ENERGY, F32>(a, c, s) : launch_t<4, 3, ENERGY, F32>(a, c, s);
+    return team_warps(a.nv.N) == 1 ? launch_t<1, 1, ENERGY, F32>(a, c, s) : launch_t<4, 3, ENERGY, F32>(a, c, s);
 }
 
 template <bool F32>
