@@ -198,6 +198,14 @@ __device__ __forceinline__ void reaction_pass(const NetView &nv, const NetSmem &
                                               float *__restrict__ J32, bool doJ)
 {
     const int N = NT > 0 ? NT : nv.N, ns = nv.ns, nr = nv.nr;
+    // The kernels with several lanes per cell round a rate and a partial before they add them.
+    // In this one variant (any size, FP64, no temperature, all reactions A + B -> C + D) the
+    // compiler would fuse the product into the sum, and the last bits would differ.
+    constexpr bool ROUND = NT == 0 && MODE == 1 && S2 && !ENERGY;
+    auto mul = [](double x, double y) {
+        if constexpr (ROUND) return __dmul_rn(x, y);
+        else return x * y;
+    };
 #pragma unroll
     for (int i = 0; i < N; ++i) LI(W, i) = 0.0;
     if (MODE == 1) {
@@ -233,7 +241,7 @@ __device__ __forceinline__ void reaction_pass(const NetView &nv, const NetSmem &
             y0q[q] = y0;
             y1q[q] = y1;
             y2q[q] = y2;
-            wq[q] = S2 ? k * (y0 * y1) : k * (y0 * y1) * y2;
+            wq[q] = S2 ? mul(k, y0 * y1) : k * (y0 * y1) * y2;
         }
 #pragma unroll
         for (int q = 0; q < kChunk; ++q) {
@@ -272,7 +280,7 @@ __device__ __forceinline__ void reaction_pass(const NetView &nv, const NetSmem &
             if (MODE == 1 && dist) {
                 const double hk = hph * k;
                 const double d2 = ENERGY ? hph * (k * (t.b[r] + t.th[r] * invT) * invT) * (y0 * y1) : 0.0;
-                scatter22<double, 5, ENERGY>(M64, N, ns, i0, i1, o0, o1, hk * y1, hk * y0, d2,
+                scatter22<double, 5, ENERGY>(M64, N, ns, i0, i1, o0, o1, mul(hk, y1), mul(hk, y0), d2,
                                              ENERGY ? dHr * invCV : 0.0, 1.0);
             } else if (MODE == 1) {
                 // M = I - h J: a reactant row gains +h dw/dy_m, a product row -h dw/dy_m,
@@ -288,8 +296,8 @@ __device__ __forceinline__ void reaction_pass(const NetView &nv, const NetSmem &
                     if (!S2 && nout > 2) LI(M64, o2 * N + m) -= hd;
                     if (ENERGY) LI(M64, ns * N + m) += q2 * hd;
                 };
-                col(i0, S2 ? hk * y1 : hk * y1 * y2);
-                if (nin > 1) col(i1, S2 ? hk * y0 : hk * y0 * y2);
+                col(i0, S2 ? mul(hk, y1) : hk * y1 * y2);
+                if (nin > 1) col(i1, S2 ? mul(hk, y0) : hk * y0 * y2);
                 if (!S2 && nin > 2) col(i2, hk * (y0 * y1));
                 if (ENERGY) {
                     const double dkh = hph * (k * (t.b[r] + t.th[r] * invT) * invT);
