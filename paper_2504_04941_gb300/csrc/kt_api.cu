@@ -1058,6 +1058,7 @@ int kt_autotune(const kt_network *net, int64_t ncells, const double *y_in, const
             kt::LaunchArgs a{};
             a.nv = net->view;
             a.o = dev_opts(base);
+            a.dt = dt;
             a.ncells = ncells;
             a.mlp = base->guess == KT_GUESS_MLP ? blob : nullptr;
             route_groups(net, blob, kt::LaunchCfg{base->form, per, 0, 0, fam, vars[vi]}, &a);

@@ -40,10 +40,16 @@ PROBE = r"""
 // out: lanes per cell (0: one cell per lane), size of the kernel, largest matrix place
 // written, first byte of the matrix, first byte behind it, element size, whether the programs
 // of that many lanes are laid out
-extern "C" int route(int N, int energy, int form, int scheme, long long ncells, int nr, const int *nin, const int *in,
-                     int *out)
+// (dt in first steps; negative: one per cell)
+extern "C" int route_dt(int N, int energy, int form, int scheme, long long ncells, double dt, int nr, const int *nin,
+                        const int *in, int *out)
 {
     kt::LaunchArgs a{};
+    const double dt_cell = dt;
+    a.dt = dt;
+    a.dt_cell = dt < 0.0 ? &dt_cell : nullptr;
+    a.o.h_init = 1.0;
+    a.o.facmax = 4.0;
     a.nv.N = N;
     a.nv.ns = N - energy;
     a.nv.nr = nr;
@@ -69,6 +75,15 @@ extern "C" int route(int N, int energy, int form, int scheme, long long ncells, 
     out[6] = kt::coop_sizes(kt::coop_nm(N, energy), f32) * 4 & a.coop_g;
     return 1;
 }
+extern "C" int route(int N, int energy, int form, int scheme, long long ncells, int nr, const int *nin, const int *in,
+                     int *out)
+{
+    for (double dt : {1e-3, 1.0, 1e6}) {
+        const int got = route_dt(N, energy, form, scheme, ncells, dt, nr, nin, in, out);
+        if (got) return got;
+    }
+    return 0;
+}
 """
 
 
@@ -85,6 +100,7 @@ def probe(tmp_path_factory):
     subprocess.run([cxx, "-std=c++17", "-O1", "-shared", "-fPIC", "-I", CSRC, "-I", os.path.join(ROOT, "include"),
                     str(src), "-o", str(so)], check=True, capture_output=True)
     lib = ctypes.CDLL(str(so))
+    lib.route_dt.argtypes = [ctypes.c_int] * 4 + [ctypes.c_longlong, ctypes.c_double, ctypes.c_int] + [ctypes.c_void_p] * 3
     lib.route.argtypes = [ctypes.c_int] * 4 + [ctypes.c_longlong, ctypes.c_int] + [ctypes.c_void_p] * 3
     return lib
 
