@@ -50,6 +50,10 @@ struct AdvArgs {
     double vr[NV];
 };
 
+// a b / s for sums whose reciprocal is subnormal.  Out of line: the division inlined under its
+// branch is computed for every slope (160^3 cells, ten species: 3.80 -> 6.36 ms).
+__device__ __noinline__ double large_quotient(double a, double b, double s) { return a / s * b; }
+
 // dx / 2 times the slope of the modified van Leer limiter from the forward and backward
 // differences a and b: min(a b / (a + b), b / 2) in magnitude (the first when |a| <= |b|),
 // zero at extrema; the uniform-grid geometric factor 2c/(c+d) is 1.
@@ -69,9 +73,9 @@ __device__ __forceinline__ double half_slope(double a, double b)
     // b / 2: one less in the exponent; below 2^-1021, where a double is the integer of its bits
     // times 2^-1074, half of that integer (ties to even)
     const double half = __longlong_as_double(ib >= 2 * bit ? bb - bit : (bb & ~m) | ((ib + ((ib >> 1) & 1)) >> 1));
-    // zero: signs differ, a zero or a NaN, or so small (2^-959) that a b underflows
     const long long is = __double_as_longlong(s) & m;
-    if (is >= 2045 * bit) q = a / s * b;   // the seed of 1/s would be subnormal: 0
+    if (__builtin_expect(is >= 2045 * bit, 0)) q = large_quotient(a, b, s);
+    // zero: signs differ, a zero or a NaN, or so small (2^-959) that a b underflows
     const bool zero = (ba ^ bb) < 0 || ia == 0 || ib == 0 || ia > inf || ib > inf || is < 64 * bit;
     return zero ? 0.0 : (ia <= ib || ia == inf ? q : half);
 }
