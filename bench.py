@@ -45,10 +45,10 @@ UNIT = "cell-integrations/s"
 # FP32 152 x 128 FMA/clk x 2 x 2.07 GHz = 80.5 TFLOP/s.
 FP64_NOMINAL_TFLOPS = 1.25
 FP32_NOMINAL_TFLOPS = 80.5
-# DRAM bytes (read + write) per cell of one launch of the chosen-form lane kernel on the
+# DRAM bytes (read + write) per cell of one launch of the chosen-form kernel on the
 # combustion network, from an ncu capture of the kernel built from the sources whose
 # hash is the key (a different build reports traffic null until it is captured again).
-LANE_TRAFFIC_BYTES_PER_CELL = {
+TRAFFIC_BYTES_PER_CELL = {
     # lean lane kernel, full interval, 8-warp blocks: 8,111,360 B read + 345,856 B written
     # (captured on sources f60b55e70311ee05; this key adds comments in include/kt.h only)
     "b6a2b16ed131dd4b": (8111360 + 345856) / 65536,
@@ -67,6 +67,15 @@ def kernel_source_hash() -> str:
     with open(os.path.join(ROOT, "include", "kt.h"), "rb") as f:
         h.update(f.read())
     return h.hexdigest()[:16]
+
+
+def kernel_name(wl, ncells: int, lane_variant: int) -> str:
+    """The kernel that integrates this workload's batch (csrc/kt_coop.cu coop_group at the
+    workloads' intervals): groups of lanes, one cell per lane, or teams of warps."""
+    if wl.network.n > 16 or wl.network.tables or wl.network.photo:
+        return "warp_kernel"
+    groups = wl.network.n == 11 if wl.network.energy else wl.network.n == 3 and ncells < 16 * 4 * 152
+    return "coop_kernel" if groups and lane_variant != 1 else "lane_kernel"
 
 
 # ------------------------------------------------------------------ work counts
@@ -298,7 +307,7 @@ def main():
     ap.add_argument("--no-cpu-baseline", action="store_true")
     ap.add_argument("--no-e2e", action="store_true")
     ap.add_argument("--lane-variant", type=int, default=None,
-                    help="fix the FP32-LU lane kernels' storage variant (kt.h KT_LANE_*) instead of tuning it")
+                    help="fix the FP32-LU small-network kernels' variant (kt.h KT_LANE_*) instead of tuning it")
     ap.add_argument("--block-warps", type=int, default=None,
                     help="fix the warps per block of the chosen form instead of tuning it")
     ap.add_argument("--cpu-cells", type=int, default=1024)
@@ -544,7 +553,7 @@ def main():
 
     if rank == 0:
         r = head
-        per_cell = LANE_TRAFFIC_BYTES_PER_CELL.get(kernel_source_hash())
+        per_cell = TRAFFIC_BYTES_PER_CELL.get(kernel_source_hash())
         traffic = (per_cell * ncells if per_cell and args.workload == 2 and head_name == "chosen"
                    else None)
         hbm_peak, hbm_src = hbm_peak_gbs()
@@ -561,7 +570,7 @@ def main():
                 "hbm_gbs": hbm_gbs, "hbm_peak_gbs": hbm_peak, "hbm_peak_source": hbm_src,
                 "hbm_frac": hbm_gbs / hbm_peak if hbm_gbs else None,
                 "kernel_source_hash": kernel_source_hash(),
-                "kernel": f"{'lane_kernel' if wl.network.n <= 16 else 'warp_kernel'} ({head_name} form)"}
+                "kernel": f"{kernel_name(wl, ncells, forms[head_name].get('lane_variant', 0))} ({head_name} form)"}
         if head_name == "chosen" and "fp32_flops_lower_bound" in r:
             roof["fp32_achieved_tflops"] = r["fp32_flops_lower_bound"] / (r["ms_per_step"] * 1e-3) / 1e12
             roof["fp32_frac"] = roof["fp32_achieved_tflops"] / p32

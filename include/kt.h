@@ -132,7 +132,9 @@ typedef struct {
     int use_graph;           /* 1: kt_integrate replays a captured CUDA graph    (0) */
     int cells_per_warp;      /* 32: the small-network kernels (<= 16 unknowns), one cell
                                 per lane or, where that is faster, per group of lanes
-                                (the same results bit for bit); 1: the large-network
+                                (the same results bit for bit; in FP32-LU form for 3
+                                isothermal unknowns and 11 with temperature under
+                                TR-BDF2, other sizes one per lane); 1: the large-network
                                 kernels, a cell per team of one or four
                                 warps (<= 96 unknowns); 0: automatic (0) */
     int schedule;            /* kt_integrate on a state with persistent = 1: 1 hands

@@ -9,7 +9,7 @@
 // are held one component per lane, and the Jacobian's entries and the elimination go over
 // the lanes too, so the chain shrinks to 165 FP64 instructions (G = 32, counted) and a
 // warp's 32 / G cells share each of them.  Combustion network, dt 1e-6 s, FP32-LU: 250 cells
-// 832 -> 58 ms (G = 32), 65,536 cells end to end 1,047 -> 723 ms (G = 8).
+// 808 -> 55 ms (G = 32), 65,536 cells end to end 1,040 -> 722 ms (G = 8).
 //
 // The results are bit for bit those of the lane-per-cell kernels (kt_lane.cuh): every
 // rate, every sum (same terms, same order, one lane per sum), every matrix entry (its

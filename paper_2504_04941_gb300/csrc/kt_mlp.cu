@@ -12,8 +12,8 @@
 // All products are mma.sync m16n8k16 BF16 x BF16 -> FP32, operands by ldmatrix.
 // What bounds it: latency (0.9 GFLOP and 0.7 MB at a batch of 4,096).  Before, a tile read
 // every weight fragment from global memory, 25 single warps summed dW over the whole batch
-// and 400 threads the biases one sample at a time: 668 us for loss and gradients at a batch of
-// 4,096, copies to the host included; now 131 us.
+// and 400 threads the biases one sample at a time: 657 us for loss and gradients at a batch of
+// 4,096, copies to the host included; now 122 us.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 

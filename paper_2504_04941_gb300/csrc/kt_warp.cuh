@@ -1217,7 +1217,7 @@ int launch_t(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
 // unknowns one warp holds a row per lane and four would mostly wait for each other
 // (32 species, dt 1e8 s, one | four warps, before the Jacobian program: 300 cells
 // 163 | 159 ms, 2,049 cells 134 | 189, 8,192 cells 207 | 475); beyond, the team is faster at
-// every size (65 unknowns, dt 1e-9 s: 1,024 cells 546 | 291 ms, with the program 251; 8,192
+// every size (65 unknowns, dt 1e-9 s: 1,024 cells 546 | 291 ms, with the program 258; 8,192
 // cells at 1e-10 s 615 | 405).
 template <bool F32, bool ENERGY>
 int launch_warp_size(const LaunchArgs &a, const LaunchCfg &c, cudaStream_t s)
