@@ -49,9 +49,8 @@ FP32_NOMINAL_TFLOPS = 80.5
 # combustion network, from an ncu capture of the kernel built from the sources whose
 # hash is the key (a different build reports traffic null until it is captured again).
 TRAFFIC_BYTES_PER_CELL = {
-    # lean lane kernel, full interval, 8-warp blocks: 8,111,360 B read + 345,856 B written
-    # (captured on sources f60b55e70311ee05; this key adds comments in include/kt.h only)
-    "b6a2b16ed131dd4b": (8111360 + 345856) / 65536,
+    # coop_kernel<11, 8>, full interval: 6,222,848 B read + 204,544 B written
+    "2c590d7f6180bfb2": (6222848 + 204544) / 65536,
 }
 
 
